@@ -292,11 +292,12 @@ lbm_status lbm_get_objective(lbm_ctx* ctx, double* J);
  * 7*n values.  Either may be null. */
 lbm_status lbm_get_adjoint(lbm_ctx* ctx, void* fstar, void* gstar, int dtype, int on_device);
 
-/* Time plain fused steps of one phase: n steps (rounded up to even) are
- * captured as a CUDA graph, replayed once untimed, then replayed between two
- * CUDA events recorded on the context's stream; writes the mean milliseconds
- * per step of the timed replay (kernel time plus the gaps between graph
- * nodes).  phase: 0 flow forward, 1 temperature forward, 2 flow adjoint,
+/* Time plain steps of one phase as a solve runs them (a launch each, or n steps
+ * in two resident launches when the lattice fits on the chip): n steps (rounded
+ * up to even) are captured as a CUDA graph, replayed once untimed, then
+ * replayed between two CUDA events recorded on the context's stream; writes
+ * the mean milliseconds per step of the timed replay (kernel time plus the
+ * gaps between graph nodes).  phase: 0 flow forward, 1 temperature forward, 2 flow adjoint,
  * 3 temperature adjoint.  The 2n steps advance that phase's state as a solve
  * would; no reduction runs.  Needs the inputs set (LBM_ERR_ORDER) and, for
  * phases 1-3, a completed lbm_forward. */
@@ -463,7 +464,9 @@ const char* lbm_last_error(void);
  * kernels use for every node and every direction e_i, both ways (x - e_i for
  * the forward pull, x + e_i for the adjoint pull), and stores in *mismatches
  * how many computed sources differ from the periodic wrap of x -/+ e_i or fall
- * outside the lattice.  stencil: 0 D2Q9, 1 D3Q19, 2 D3Q7 (temperature).
+ * outside the lattice.  For a lattice small enough for resident launches the
+ * count includes the populations that such a launch would send to another word
+ * than their receiver reads, under every set of symmetry planes.  stencil: 0 D2Q9, 1 D3Q19, 2 D3Q7 (temperature).
  * Errors: LBM_ERR_ARG (null pointer, bad sizes, more than 2^24 nodes). */
 lbm_status lbm_check_addressing(int stencil, int nx, int ny, int nz, long long* mismatches);
 

@@ -359,11 +359,9 @@ __device__ __forceinline__ void block_partials(double (&v)[NV], double* __restri
 //   offset populations h (w_i = w_opp(i), sum_{e.n=0} e w = 0)
 // ---------------------------------------------------------------------------
 template <class L, typename R>
-__device__ __forceinline__ void zou_he(R (&f)[L::Q], int type, int code, const R* __restrict__ bc, R rho0) {
+__device__ __forceinline__ void zou_he_along(R (&f)[L::Q], int type, int n0, int n1, int n2,
+                                             const R* __restrict__ bc, R rho0) {
     using X = Ex<R>;
-    const int ax = code >> 1;
-    const int sg = (code & 1) ? -1 : 1;
-    const int n0 = ax == 0 ? sg : 0, n1 = ax == 1 ? sg : 0, n2 = ax == 2 ? sg : 0;
     R K0 = 0, Km = 0, S0 = 0, S1 = 0, S2 = 0;
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) {
@@ -406,6 +404,32 @@ __device__ __forceinline__ void zou_he(R (&f)[L::Q], int type, int code, const R
     }
 }
 
+// call fn(n0, n1, n2) with the inward normal of a code.  FIXED: one copy of fn
+// per normal, its components constants (an operator of a fifth of the
+// instructions, for kernels in which a step waits for its slowest warp); else
+// one copy for all (less code and fewer registers in the one-step kernels,
+// where the few open nodes cost nothing).
+template <class L, bool FIXED, class Fn>
+__device__ __forceinline__ void with_normal(int code, Fn fn) {
+    if (!FIXED) {
+        const int ax = code >> 1;
+        const int sg = (code & 1) ? -1 : 1;
+        fn(ax == 0 ? sg : 0, ax == 1 ? sg : 0, ax == 2 ? sg : 0);
+        return;
+    }
+    if (code == 0) fn(1, 0, 0);
+    else if (code == 1) fn(-1, 0, 0);
+    else if (code == 2) fn(0, 1, 0);
+    else if (L::Q == 9 || code == 3) fn(0, -1, 0);
+    else if (code == 4) fn(0, 0, 1);
+    else fn(0, 0, -1);
+}
+
+template <class L, bool FIXED = false, typename R>
+__device__ __forceinline__ void zou_he(R (&f)[L::Q], int type, int code, const R* __restrict__ bc, R rho0) {
+    with_normal<L, FIXED>(code, [&](int n0, int n1, int n2) { zou_he_along<L>(f, type, n0, n1, n2, bc, rho0); });
+}
+
 // adjoint boundary operator f* = B^T f*_C for a Zou-He node:
 //   unknown j           : 0
 //   e_j.n < 0           : c_j + c_opp(j)              (- 2P at PRES)
@@ -413,11 +437,8 @@ __device__ __forceinline__ void zou_he(R (&f)[L::Q], int type, int code, const R
 // with M = sum_{k in U} e_k c_k and P = sum_{k in U} 6 w_k c_k.  In D2Q9 this is
 // Eq. 59 (left velocity inlet) and Eq. 60 (bottom fixed-density outlet).
 template <class L, typename R>
-__device__ __forceinline__ void zou_he_adjoint(R (&c)[L::Q], int type, int code) {
+__device__ __forceinline__ void zou_he_adjoint_along(R (&c)[L::Q], int type, int n0, int n1, int n2) {
     using X = Ex<R>;
-    const int ax = code >> 1;
-    const int sg = (code & 1) ? -1 : 1;
-    const int n0 = ax == 0 ? sg : 0, n1 = ax == 1 ? sg : 0, n2 = ax == 2 ? sg : 0;
     R M0 = 0, M1 = 0, M2 = 0, P = 0;
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) {
@@ -444,6 +465,11 @@ __device__ __forceinline__ void zou_he_adjoint(R (&c)[L::Q], int type, int code)
         const int d = L::cx(i) * n0 + L::cy(i) * n1 + L::cz(i) * n2;
         if (d > 0) c[i] = R(0);
     }
+}
+
+template <class L, bool FIXED = false, typename R>
+__device__ __forceinline__ void zou_he_adjoint(R (&c)[L::Q], int type, int code) {
+    with_normal<L, FIXED>(code, [&](int n0, int n1, int n2) { zou_he_adjoint_along<L>(c, type, n0, n1, n2); });
 }
 
 template <class L, typename R>
@@ -620,10 +646,12 @@ struct FwdMinBlocks {
     static constexpr int value = L::Q != 19 ? 1 : (sizeof(T) == 2 ? 6 : (sizeof(T) == 4 ? 5 : 1));
 };
 
+// bail (or null): a reducing step that finds the flag set leaves everything as it is
 template <class L, typename T, typename TA, typename R, bool REDUCE, bool MIRROR>
-__global__ void __launch_bounds__(256, (FwdMinBlocks<L, T>::value)) k_flow_step(FlowArgs<T, TA, R> a) {
+__global__ void __launch_bounds__(256, (FwdMinBlocks<L, T>::value)) k_flow_step(FlowArgs<T, TA, R> a, const int* bail) {
     pdl_launch_dependents();
     pdl_wait();
+    if (REDUCE && bail && *bail) return;
     const Cell c = this_cell(a.nx, a.ny);
     double acc[2] = {0.0, 0.0};
     if (c.active) flow_step_node<L, T, TA, R, REDUCE, MIRROR>(a, c, acc);
@@ -800,11 +828,10 @@ struct AdjMinBlocks {
 // adjoint collision at a non-wall node, in place (Eq. 63-65): f*_C,i =
 // (1 - 1/tau) f*_S,i + (1/tau) sum_m (d f^eq_m / d f_i) f*_S,m
 // [- dJ/df_i = 1/(3 N_in) at an inlet node when src] [+ thermal coupling]
-template <class L, typename T, typename TA, typename R, bool THERMAL, bool CPL_RT>
-__device__ __forceinline__ void adjoint_collide(const FlowArgs<T, TA, R>& a, long long n, bool src, R (&s)[L::Q]) {
+template <class L, typename R>
+__device__ __forceinline__ void adjoint_collide_values(R om, int model, R src_in, bool src, R g, R u0, R u1, R u2,
+                                                       R v0, R v1, R v2, R (&s)[L::Q]) {
     using X = Ex<R>;
-    const R g = a.gamma[n];
-    const R u0 = a.u[n], u1 = a.u[a.np + n], u2 = a.u[2 * a.np + n];
     AdjMoments<L, R> m;
     m.compute(s);
     const R Qu0 = X::fma(m.Q02, u2, X::fma(m.Q01, u1, X::mul(m.Q00, u0)));
@@ -812,23 +839,16 @@ __device__ __forceinline__ void adjoint_collide(const FlowArgs<T, TA, R>& a, lon
     const R Qu2 = X::fma(m.Q22, u2, X::fma(m.Q12, u1, X::mul(m.Q02, u0)));
     // sum_m (d f^eq_m / d f_i) f*_m = A + e_i . w
     const R c1 = X::mul(R(3), g);
-    const R c2 = a.model == 0 ? X::mul(X::mul(R(9), g), g) : X::mul(R(9), g);
-    const R c3 = a.model == 0 ? X::mul(c1, g) : c1;
+    const R c2 = model == 0 ? X::mul(X::mul(R(9), g), g) : X::mul(R(9), g);
+    const R c3 = model == 0 ? X::mul(c1, g) : c1;
     const R c3A = X::mul(c3, m.A);
     R w0 = X::fma(-c3A, u0, X::fma(c2, Qu0, X::mul(c1, m.M0)));
     R w1 = X::fma(-c3A, u1, X::fma(c2, Qu1, X::mul(c1, m.M1)));
     R w2 = X::fma(-c3A, u2, X::fma(c2, Qu2, X::mul(c1, m.M2)));
-    const R om = a.omega;
     R base = X::mul(om, m.A);
-    if (src) base = X::sub(base, a.src_in);
+    if (src) base = X::sub(base, src_in);
     // the coupling term enters through the same fused operation whether
     // it is present or zero, so every kernel variant rounds alike
-    R v0 = 0, v1 = 0, v2 = 0;
-    if (THERMAL || (CPL_RT && a.cpl != nullptr)) {
-        v0 = a.cpl[n];
-        v1 = a.cpl[a.np + n];
-        v2 = a.cpl[2 * a.np + n];
-    }
     w0 = X::fma(om, w0, v0);
     w1 = X::fma(om, w1, v1);
     w2 = X::fma(om, w2, v2);
@@ -842,6 +862,18 @@ __device__ __forceinline__ void adjoint_collide(const FlowArgs<T, TA, R>& a, lon
         s[i] = X::fma(om1, s[i], X::add(base, ew));
         s[j] = X::fma(om1, s[j], X::sub(base, ew));
     }
+}
+
+template <class L, typename T, typename TA, typename R, bool THERMAL, bool CPL_RT>
+__device__ __forceinline__ void adjoint_collide(const FlowArgs<T, TA, R>& a, long long n, bool src, R (&s)[L::Q]) {
+    R v0 = 0, v1 = 0, v2 = 0;
+    if (THERMAL || (CPL_RT && a.cpl != nullptr)) {
+        v0 = a.cpl[n];
+        v1 = a.cpl[a.np + n];
+        v2 = a.cpl[2 * a.np + n];
+    }
+    adjoint_collide_values<L, R>(a.omega, a.model, a.src_in, src, a.gamma[n], a.u[n], a.u[a.np + n],
+                                 a.u[2 * a.np + n], v0, v1, v2, s);
 }
 
 template <class L, typename T, typename TA, typename R, bool REDUCE, bool THERMAL, bool CPL_RT = false,
@@ -870,9 +902,10 @@ __device__ __forceinline__ void flow_adjoint_node(const FlowArgs<T, TA, R>& a, c
 
 template <class L, typename T, typename TA, typename R, bool REDUCE, bool THERMAL, bool MIRROR>
 __global__ void __launch_bounds__(256, (AdjMinBlocks<L, R, REDUCE, THERMAL>::value))
-    k_flow_adjoint(FlowArgs<T, TA, R> a) {
+    k_flow_adjoint(FlowArgs<T, TA, R> a, const int* bail) {
     pdl_launch_dependents();
     pdl_wait();
+    if (REDUCE && bail && *bail) return;
     const Cell c = this_cell(a.nx, a.ny);
     double acc[1] = {0.0};
     if (c.active) flow_adjoint_node<L, T, TA, R, REDUCE, THERMAL, false, MIRROR>(a, c, acc);
@@ -1081,12 +1114,10 @@ __device__ __forceinline__ int thermal_pull(const ThermArgs<T, TA, R>& a, const 
 
 // temperature collision at a non-wall node with the heat source w_k Q,
 // Q = beta_max (1 - gamma)(1 - T) (Eq. 69, 71), in place; returns Q
-template <typename T, typename TA, typename R>
-__device__ __forceinline__ R thermal_collide(const ThermArgs<T, TA, R>& a, R (&g)[7], R tem, R gam, R u0, R u1,
-                                             R u2) {
+template <typename R>
+__device__ __forceinline__ R thermal_collide_values(R beta, R (&g)[7], R tem, R om, R gam, R u0, R u1, R u2) {
     using X = Ex<R>;
-    const R qs = X::mul(X::mul(a.beta, X::sub(R(1), gam)), X::sub(R(1), tem));
-    const R om = R(1) / tau_g<R>(gam, a.kappa_f, a.k_ratio);
+    const R qs = X::mul(X::mul(beta, X::sub(R(1), gam)), X::sub(R(1), tem));
     const R g4 = X::mul(R(4), gam);
 #pragma unroll
     for (int k = 1; k < 7; ++k) {
@@ -1101,6 +1132,12 @@ __device__ __forceinline__ R thermal_collide(const ThermArgs<T, TA, R>& a, R (&g
     for (int k = 2; k < 7; ++k) moved = X::add(moved, g[k]);
     g[0] = X::sub(X::add(tem, qs), moved);
     return qs;
+}
+
+template <typename T, typename TA, typename R>
+__device__ __forceinline__ R thermal_collide(const ThermArgs<T, TA, R>& a, R (&g)[7], R tem, R gam, R u0, R u1,
+                                             R u2) {
+    return thermal_collide_values<R>(a.beta, g, tem, R(1) / tau_g<R>(gam, a.kappa_f, a.k_ratio), gam, u0, u1, u2);
 }
 
 // one temperature step at a node; the reducing step also sums T (residual,
@@ -1157,9 +1194,10 @@ __global__ void __launch_bounds__(256) k_thermal_collide_initial(ThermArgs<T, TA
 }
 
 template <typename T, typename TA, typename R, bool REDUCE, bool MIRROR>
-__global__ void __launch_bounds__(256) k_thermal_step(ThermArgs<T, TA, R> a) {
+__global__ void __launch_bounds__(256) k_thermal_step(ThermArgs<T, TA, R> a, const int* bail) {
     pdl_launch_dependents();
     pdl_wait();
+    if (REDUCE && bail && *bail) return;
     const Cell c = this_cell(a.nx, a.ny);
     double acc[2] = {0.0, 0.0};
     if (c.active) thermal_step_node<T, TA, R, REDUCE, MIRROR>(a, c, acc);
@@ -1223,42 +1261,51 @@ __device__ __forceinline__ void thermal_pull_adjoint(const ThermArgs<T, TA, R>& 
     for (int k = 0; k < 7; ++k, p += a.np) s[k] = Pop<TA>::ld(p, nbr_offset<D3Q7>(o, k, +1), R(0)) * a.ascale;
 }
 
+// collision and boundary of the thermal adjoint at one node, in place; true at
+// an outflow node, whose unknown's adjoint before the boundary is ckn
+template <typename R>
+__device__ __forceinline__ bool thermal_adjoint_update(R src_q, R src_T, R beta, int fl, R om, R gam, R u0, R u1, R u2,
+                                                       R (&s)[7], R& ckn) {
+    const int type = fl & 7;
+    if (type == WALL) {
+        bounce<D3Q7>(s);
+        return false;
+    }
+    // -dJ/dg_l: mean-T objective and heat-generation objective (Eq. 72)
+    const R src = Ex<R>::fma(src_q, Ex<R>::sub(R(1), gam), src_T);
+    thermal_adjoint_collide<R>(s, gam, u0, u1, u2, om, src, beta);
+    if (type < VEL) return false;
+    const int kn = ((fl >> 3) & 7) + 1;
+    ckn = 0;
+    R en = 0;
+#pragma unroll
+    for (int k = 1; k < 7; ++k)
+        if (k == kn) {
+            ckn = s[k];
+            en = ecomp<R>(k, u0, u1, u2);
+        }
+    const bool outflow = !(type == VEL || (fl & HEAT_BIT));
+    R coef = R(-1);
+    if (outflow) {
+        const R wa = Ex<R>::mul(R(0.125), Ex<R>::fma(Ex<R>::mul(R(4), gam), en, R(1)));
+        coef = wa / Ex<R>::sub(R(1), wa);
+    }
+#pragma unroll
+    for (int k = 0; k < 7; ++k) s[k] = (k == kn) ? R(0) : Ex<R>::fma(coef, ckn, s[k]);
+    return outflow;
+}
+
 template <typename T, typename TA, typename R, bool REDUCE, bool MIRROR = true>
 __device__ __forceinline__ void thermal_adjoint_node(const ThermArgs<T, TA, R>& a, const Cell& c, double (&acc)[1]) {
     R s[7];
     thermal_pull_adjoint<MIRROR>(a, c, s);
     const int fl = a.flags[c.n];
     const int type = fl & 7;
-    if (type == WALL) {
-        bounce<D3Q7>(s);
-    } else {
-        const R gam = a.gamma[c.n];
-        const R u0 = a.u[c.n], u1 = a.u[a.np + c.n], u2 = a.u[2 * a.np + c.n];
-        const R om = R(1) / tau_g<R>(gam, a.kappa_f, a.k_ratio);
-        // -dJ/dg_l: mean-T objective and heat-generation objective (Eq. 72)
-        const R src = Ex<R>::fma(a.src_q, Ex<R>::sub(R(1), gam), a.src_T);
-        thermal_adjoint_collide<R>(s, gam, u0, u1, u2, om, src, a.beta);
-        if (type >= VEL) {
-            const int kn = ((fl >> 3) & 7) + 1;
-            R ckn = 0, en = 0;
-#pragma unroll
-            for (int k = 1; k < 7; ++k)
-                if (k == kn) {
-                    ckn = s[k];
-                    en = ecomp<R>(k, u0, u1, u2);
-                }
-            R coef;
-            if (type == VEL || (fl & HEAT_BIT)) {
-                coef = R(-1);
-            } else {
-                const R wa = Ex<R>::mul(R(0.125), Ex<R>::fma(Ex<R>::mul(R(4), gam), en, R(1)));
-                coef = wa / Ex<R>::sub(R(1), wa);
-                a.gcn[c.n] = ckn;
-            }
-#pragma unroll
-            for (int k = 0; k < 7; ++k) s[k] = (k == kn) ? R(0) : Ex<R>::fma(coef, ckn, s[k]);
-        }
-    }
+    const R gam = a.gamma[c.n];
+    R ckn;
+    if (thermal_adjoint_update<R>(a.src_q, a.src_T, a.beta, fl, R(1) / tau_g<R>(gam, a.kappa_f, a.k_ratio), gam,
+                                  a.u[c.n], a.u[a.np + c.n], a.u[2 * a.np + c.n], s, ckn))
+        a.gcn[c.n] = ckn;
     const R inv = R(1) / a.ascale;
 #pragma unroll
     for (int k = 0; k < 7; ++k) Pop<TA>::st(a.aout, (size_t)k * a.np + c.n, s[k] * inv, R(0));
@@ -1271,9 +1318,10 @@ __device__ __forceinline__ void thermal_adjoint_node(const ThermArgs<T, TA, R>& 
 }
 
 template <typename T, typename TA, typename R, bool REDUCE, bool MIRROR>
-__global__ void __launch_bounds__(256) k_thermal_adjoint(ThermArgs<T, TA, R> a) {
+__global__ void __launch_bounds__(256) k_thermal_adjoint(ThermArgs<T, TA, R> a, const int* bail) {
     pdl_launch_dependents();
     pdl_wait();
+    if (REDUCE && bail && *bail) return;
     const Cell c = this_cell(a.nx, a.ny);
     double acc[1] = {0.0};
     if (c.active) thermal_adjoint_node<T, TA, R, REDUCE, MIRROR>(a, c, acc);
@@ -1495,10 +1543,16 @@ __global__ void __launch_bounds__(256) k_batch_finalize(const int* __restrict__ 
 }
 
 // deterministic second stage of every reduction: one block sums the per-block
-// partials in a fixed order
+// partials in a fixed order; after a block with a resident launch (sync not
+// null: its step counter and error flag) also passes the error flag on in
+// out[2] and moves the counter past the block's `steps` steps
 template <int NV>
 __global__ void __launch_bounds__(256) k_finalize(const double* __restrict__ partials, long long nblocks,
-                                                  double* __restrict__ out) {
+                                                  double* __restrict__ out, unsigned* __restrict__ sync, int steps) {
+    if (sync && threadIdx.x == 0) {
+        out[2] = (double)sync[1];
+        sync[0] += (unsigned)steps;
+    }
     double s[NV];
 #pragma unroll
     for (int k = 0; k < NV; ++k) s[k] = 0.0;

@@ -96,8 +96,8 @@ inline dim3 flat_grid(long long np) { return dim3((unsigned)((np + 255) / 256));
 
 // launch a step kernel as a programmatic dependent of the previous kernel in
 // the stream (the kernel waits for it with griddepcontrol.wait)
-template <typename Arg>
-void launch_pdl(void (*kernel)(Arg), const Geom& g, cudaStream_t s, const Arg& a) {
+template <typename... Args>
+void launch_pdl(void (*kernel)(Args...), const Geom& g, cudaStream_t s, const Args&... a) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = g.grid;
     cfg.blockDim = g.block;
@@ -108,7 +108,7 @@ void launch_pdl(void (*kernel)(Arg), const Geom& g, cudaStream_t s, const Arg& a
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, a);
+    cudaLaunchKernelEx(&cfg, kernel, a...);
 }
 
 template <class L, int S, bool M>
@@ -130,13 +130,13 @@ void flow_dispatch_m(FlowOp op, const FlowLaunch& l, const Geom& g, cudaStream_t
                     break;
                 }
             }
-            launch_pdl(k_flow_step<L, T, TA, R, false, M>, g, s, a);
+            launch_pdl(k_flow_step<L, T, TA, R, false, M>, g, s, a, l.bail);
             break;
-        case FOP_STEP_RED: launch_pdl(k_flow_step<L, T, TA, R, true, M>, g, s, a); break;
-        case FOP_ADJ: launch_pdl(k_flow_adjoint<L, T, TA, R, false, false, M>, g, s, a); break;
-        case FOP_ADJ_RED: launch_pdl(k_flow_adjoint<L, T, TA, R, true, false, M>, g, s, a); break;
-        case FOP_ADJ_T: launch_pdl(k_flow_adjoint<L, T, TA, R, false, true, M>, g, s, a); break;
-        case FOP_ADJ_T_RED: launch_pdl(k_flow_adjoint<L, T, TA, R, true, true, M>, g, s, a); break;
+        case FOP_STEP_RED: launch_pdl(k_flow_step<L, T, TA, R, true, M>, g, s, a, l.bail); break;
+        case FOP_ADJ: launch_pdl(k_flow_adjoint<L, T, TA, R, false, false, M>, g, s, a, l.bail); break;
+        case FOP_ADJ_RED: launch_pdl(k_flow_adjoint<L, T, TA, R, true, false, M>, g, s, a, l.bail); break;
+        case FOP_ADJ_T: launch_pdl(k_flow_adjoint<L, T, TA, R, false, true, M>, g, s, a, l.bail); break;
+        case FOP_ADJ_T_RED: launch_pdl(k_flow_adjoint<L, T, TA, R, true, true, M>, g, s, a, l.bail); break;
         case FOP_SENS: k_flow_sens<L, T, TA, R, false, M><<<g.grid, g.block, 0, s>>>(a); break;
         case FOP_SENS_T: k_flow_sens<L, T, TA, R, true, M><<<g.grid, g.block, 0, s>>>(a); break;
         case FOP_ADJ_CONT:
@@ -173,10 +173,10 @@ void therm_dispatch_m(ThermOp op, const ThermLaunch& l, const Geom& g, cudaStrea
     switch (op) {
         case TOP_INIT_G: k_thermal_init<T, TA, R><<<flat_grid(l.np), 256, 0, s>>>(a, 0); break;
         case TOP_INIT_A: k_thermal_init<T, TA, R><<<flat_grid(l.np), 256, 0, s>>>(a, 1); break;
-        case TOP_STEP: launch_pdl(k_thermal_step<T, TA, R, false, M>, g, s, a); break;
-        case TOP_STEP_RED: launch_pdl(k_thermal_step<T, TA, R, true, M>, g, s, a); break;
-        case TOP_ADJ: launch_pdl(k_thermal_adjoint<T, TA, R, false, M>, g, s, a); break;
-        case TOP_ADJ_RED: launch_pdl(k_thermal_adjoint<T, TA, R, true, M>, g, s, a); break;
+        case TOP_STEP: launch_pdl(k_thermal_step<T, TA, R, false, M>, g, s, a, l.bail); break;
+        case TOP_STEP_RED: launch_pdl(k_thermal_step<T, TA, R, true, M>, g, s, a, l.bail); break;
+        case TOP_ADJ: launch_pdl(k_thermal_adjoint<T, TA, R, false, M>, g, s, a, l.bail); break;
+        case TOP_ADJ_RED: launch_pdl(k_thermal_adjoint<T, TA, R, true, M>, g, s, a, l.bail); break;
         case TOP_COUPLING: k_thermal_coupling<T, TA, R, M><<<g.grid, g.block, 0, s>>>(a); break;
         case TOP_COLLIDE_INIT: k_thermal_collide_initial<T, TA, R><<<g.grid, g.block, 0, s>>>(a); break;
     }

@@ -37,6 +37,7 @@ struct FlowLaunch {
     double omega, rho0, src_in, ascale;
     int model;
     int mirror;
+    const int* bail;
 };
 
 struct ThermLaunch {
@@ -57,6 +58,7 @@ struct ThermLaunch {
     long long np;
     double rho0, kappa_f, k_ratio, q, T0, src_T, ascale, beta, src_q;
     int mirror;
+    const int* bail;
 };
 
 enum FlowOp {
@@ -78,6 +80,42 @@ enum FlowOp {
 enum ThermOp { TOP_INIT_G = 0, TOP_INIT_A, TOP_STEP, TOP_STEP_RED, TOP_ADJ, TOP_ADJ_RED, TOP_COUPLING,
                TOP_COLLIDE_INIT };
 
+// Resident launches (lbm_resident.cuh): the lattice cut into px x py x pz boxes
+// of at most bx x by x bz nodes, one block each.
+struct ResGeom {
+    int nx, ny, nz, px, py, pz, bx, by, bz;
+    int pitch;        // shared-memory slots between rows (odd: a column of nodes meets every bank)
+    int cap;          // node places: pitch by bz (Q populations each)
+    int silent;       // threads that do not exchange (whole warps; the others come last)
+    int words;        // words of an exchanging thread, at most
+    int list;         // places of the node lists
+    int aux_at;       // byte offset of the per-node constants
+    int word_at;      // byte offset of the list of words
+    int inbox;        // words of one box's inbox
+    long long parity; // words of all inboxes (two sets alternate)
+};
+constexpr int kResThreads(size_t real) { return real == 8 ? 384 : 1024; }  // threads of an SM's blocks
+constexpr int kResHead = 1536;  // bytes of tables at the start of the shared memory
+struct ResPlan {
+    ResGeom g;
+    int threads;
+    int per_sm;       // blocks on an SM
+    size_t smem;
+    size_t inbox_bytes;
+    bool ok;
+};
+enum ResPhase { RP_FLOW = 0, RP_THERM, RP_ADJ, RP_TADJ, RP_ADJ_T };
+// cut of a lattice for a phase (ok = false: it does not fit on the chip); a
+// function of the sizes alone, for the 152 SMs of a GB300
+ResPlan resident_plan(int stencil, int storage, ResPhase ph, int nx, int ny, int nz);
+// `steps` plain steps of a phase in one cooperative launch: reads fin / ain /
+// gin, writes fout / aout / gout.  base: step numbers of the words start here;
+// err is set when a wait gave up.
+cudaError_t resident_flow(int stencil, int storage, ResPhase ph, const FlowLaunch& a, const ResPlan& p, void* inboxes,
+                          const unsigned* base, int* err, int steps, cudaStream_t s);
+cudaError_t resident_thermal(int storage, ResPhase ph, const ThermLaunch& a, const ResPlan& p, void* inboxes,
+                             const unsigned* base, int* err, int steps, cudaStream_t s);
+
 // storage codes follow lbm_storage; stencil codes follow lbm_stencil
 cudaError_t flow_launch(int stencil, int storage, FlowOp op, const FlowLaunch& a, const Geom& g,
                         cudaStream_t s);
@@ -86,9 +124,13 @@ cudaError_t thermal_launch(int storage, ThermOp op, const ThermLaunch& a, const 
 // host run of the kernels' pull addressing over every node (stencil 0 D2Q9,
 // 1 D3Q19, 2 D3Q7): the number of wrong or out-of-range sources
 long long addressing_mismatches(int stencil, int nx, int ny, int nz);
+// host run of the resident launches' exchange over every border node, for every
+// set of symmetry planes (stencils as above): words sent elsewhere than they are
+// read, or outside the inboxes
+long long resident_mismatches(int stencil, int nx, int ny, int nz);
 
 cudaError_t finalize_launch(const double* partials, long long nblocks, int nv, double* out,
-                            cudaStream_t s);
+                            cudaStream_t s, unsigned* sync = nullptr, int steps = 0);
 // element conversion between float/double buffers (device to device)
 cudaError_t convert_launch(const void* src, int src_f64, void* dst, int dst_f64, long long n,
                            cudaStream_t s);

@@ -91,11 +91,11 @@ long long addressing_mismatches(int stencil, int nx, int ny, int nz) {
 }
 
 cudaError_t finalize_launch(const double* partials, long long nblocks, int nv, double* out,
-                            cudaStream_t s) {
+                            cudaStream_t s, unsigned* sync, int steps) {
     if (nv == 1)
-        k_finalize<1><<<1, 256, 0, s>>>(partials, nblocks, out);
+        k_finalize<1><<<1, 256, 0, s>>>(partials, nblocks, out, sync, steps);
     else
-        k_finalize<2><<<1, 256, 0, s>>>(partials, nblocks, out);
+        k_finalize<2><<<1, 256, 0, s>>>(partials, nblocks, out, sync, steps);
     return cudaGetLastError();
 }
 

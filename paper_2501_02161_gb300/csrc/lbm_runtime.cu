@@ -2,9 +2,11 @@
 // convergence loops and result read-back.
 //
 // Each solve phase runs in blocks of K steps.  A block is captured once as a
-// CUDA graph (K-1 plain fused steps, one reducing step, the deterministic
-// finalize kernel and the copy of the sums to pinned host memory) and then
-// replayed, so a block costs one graph launch and one host synchronisation.
+// CUDA graph (K-1 plain steps, one reducing step, the deterministic finalize
+// kernel and the copy of the sums to pinned host memory) and then replayed, so
+// a block costs one graph launch and one host synchronisation.  The plain
+// steps of a lattice that fits on the chip are one resident launch
+// (lbm_resident.cuh), those of a larger one a launch each.
 // The residual |I(t) - I(t-K)| / |I(t)| is evaluated on the host from the FP64
 // sums (Sec. 3.1, Fig. 8 text).
 #include <cuda_runtime.h>
@@ -15,6 +17,7 @@
 #include <cstring>
 #include <algorithm>
 #include <map>
+#include <mutex>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -84,6 +87,12 @@ struct lbm_ctx {
     double* partials = nullptr;
     double* dres = nullptr;
     double* hres = nullptr;  // pinned, 4 doubles
+    ResPlan plan[4] = {};    // per phase: how its lattice is cut for a resident launch
+    void* inbox = nullptr;   // words exchanged by resident launches
+    unsigned* sync = nullptr;  // their step counter and error flag
+    size_t inbox_bytes = 0;
+    unsigned long long tags = 0;  // step numbers used since the counter was cleared
+    bool resident = false;
 
     Geom geom{};
     lbm_params prm{0.6, 1.0, 0, 0.0, 1.0, 0.0, 0.0, 0.0};
@@ -98,7 +107,7 @@ struct lbm_ctx {
     double J() const { return J_p + (thermal ? J_T + J_Q : 0.0); }
     double last_I[4] = {0, 0, 0, 0};
 
-    std::map<std::tuple<int, int, int>, cudaGraphExec_t> graphs;
+    std::map<std::tuple<int, int, int, bool>, cudaGraphExec_t> graphs;
     std::vector<uint8_t> hflags;   // host copy of the flags (per-face boundary values)
     int mirror = 0;                // axes with symmetry planes (lbm_set_symmetry)
     int adj_scheme = LBM_ADJOINT_DISCRETE;  // lbm_set_adjoint_scheme
@@ -114,6 +123,20 @@ namespace {
 // a destroyed context stops counting against its batch's memory budget
 void batch_forget(lbm_batch* b, lbm_ctx* c);
 
+// the cuts of a lattice's phases (out: PH_* order) and the bytes their inboxes need
+size_t resident_plans(int stencil, int nx, int ny, int nz, int storage, bool thermal, ResPlan (&out)[4]) {
+    out[PH_FLOW] = resident_plan(stencil, storage, RP_FLOW, nx, ny, nz);
+    out[PH_ADJ] = resident_plan(stencil, storage, thermal ? RP_ADJ_T : RP_ADJ, nx, ny, nz);
+    if (thermal) {
+        out[PH_THERM] = resident_plan(stencil, storage, RP_THERM, nx, ny, nz);
+        out[PH_TADJ] = resident_plan(stencil, storage, RP_TADJ, nx, ny, nz);
+    }
+    size_t bytes = 0;
+    for (const ResPlan& p : out)
+        if (p.ok) bytes = std::max(bytes, p.inbox_bytes);
+    return bytes;
+}
+
 void* dalloc(size_t bytes, cudaError_t* err) {
     void* p = nullptr;
     cudaError_t e = cudaMalloc(&p, bytes ? bytes : 16);
@@ -125,7 +148,7 @@ void free_all(lbm_ctx* c) {
     c->drop_graphs();
     void* bufs[] = {c->f[0], c->f[1], c->fa[0], c->fa[1], c->g[0], c->g[1], c->ga[0], c->ga[1],
                     c->flags, c->gamma, c->bc, c->u, c->rho, c->T, c->gpost, c->cpl, c->sT,
-                    c->gcn, c->sens, c->partials, c->dres};
+                    c->gcn, c->sens, c->partials, c->dres, c->inbox};
     for (void* p : bufs)
         if (p) cudaFree(p);
     if (c->hres) cudaFreeHost(c->hres);
@@ -203,14 +226,17 @@ int phase_nv(int ph) { return ph == PH_FLOW || ph == PH_THERM ? 2 : 1; }
 
 // enqueue one step of a phase on stream s; the reducing variant writes the
 // per-block partial sums (and the fields of the post-boundary state)
-cudaError_t enqueue_step(lbm_ctx* c, int ph, bool reduce, cudaStream_t s) {
+// after_resident: the step follows a resident launch and is left out when that gave up
+cudaError_t enqueue_step(lbm_ctx* c, int ph, bool reduce, cudaStream_t s, bool after_resident = false) {
     cudaError_t e = cudaSuccess;
+    const int* bail = after_resident ? (const int*)(c->sync + 1) : nullptr;
     if (ph == PH_FLOW) {
         FlowLaunch a = flow_base(c);
         a.fin = c->f[c->fcur];
         a.fout = c->f[1 - c->fcur];
         a.out0 = c->rho;
         a.out1 = c->u;
+        a.bail = bail;
         e = flow_launch(c->stencil, c->storage, reduce ? FOP_STEP_RED : FOP_STEP, a, c->geom, s);
         c->fcur ^= 1;
     } else if (ph == PH_THERM) {
@@ -219,12 +245,14 @@ cudaError_t enqueue_step(lbm_ctx* c, int ph, bool reduce, cudaStream_t s) {
         a.gout = c->g[1 - c->gcur];
         a.out0 = c->T;
         a.out1 = c->gpost;
+        a.bail = bail;
         e = thermal_launch(c->storage, reduce ? TOP_STEP_RED : TOP_STEP, a, c->geom, s);
         c->gcur ^= 1;
     } else if (ph == PH_ADJ) {
         FlowLaunch a = flow_base(c);
         a.ain = c->fa[c->facur];
         a.aout = c->fa[1 - c->facur];
+        a.bail = bail;
         FlowOp op = c->thermal ? (reduce ? FOP_ADJ_T_RED : FOP_ADJ_T) : (reduce ? FOP_ADJ_RED : FOP_ADJ);
         if (c->adj_scheme == LBM_ADJOINT_CONTINUOUS) op = reduce ? FOP_ADJ_CONT_RED : FOP_ADJ_CONT;
         e = flow_launch(c->stencil, c->storage, op, a, c->geom, s);
@@ -233,6 +261,7 @@ cudaError_t enqueue_step(lbm_ctx* c, int ph, bool reduce, cudaStream_t s) {
         ThermLaunch a = therm_base(c);
         a.ain = c->ga[c->gacur];
         a.aout = c->ga[1 - c->gacur];
+        a.bail = bail;
         e = thermal_launch(c->storage, reduce ? TOP_ADJ_RED : TOP_ADJ, a, c->geom, s);
         c->gacur ^= 1;
     }
@@ -243,26 +272,81 @@ int& parity_of(lbm_ctx* c, int ph) {
     return ph == PH_FLOW ? c->fcur : (ph == PH_THERM ? c->gcur : (ph == PH_ADJ ? c->facur : c->gacur));
 }
 
-// enqueue a block of k steps ending with a reduction, the finalize kernel and
-// the copy of the sums to c->hres
-cudaError_t enqueue_block(lbm_ctx* c, int ph, int k, cudaStream_t s) {
-    cudaError_t e = cudaSuccess;
-    for (int i = 0; i < k && e == cudaSuccess; ++i) e = enqueue_step(c, ph, i == k - 1, s);
-    if (e != cudaSuccess) return e;
-    e = finalize_launch(c->partials, c->geom.nblocks, phase_nv(ph), c->dres, s);
-    if (e != cudaSuccess) return e;
-    return cudaMemcpyAsync(c->hres, c->dres, sizeof(double) * phase_nv(ph), cudaMemcpyDeviceToHost, s);
+// A resident launch beats a launch per step from a handful of steps on (its
+// set-up and the global passes at its ends cost about three steps).
+constexpr int kResidentMinSteps = 6;
+
+bool resident_fits(const lbm_ctx* c, int ph, int steps) {
+    return c->resident && c->plan[ph].ok && steps >= kResidentMinSteps &&
+           !(ph == PH_ADJ && c->adj_scheme == LBM_ADJOINT_CONTINUOUS);
 }
 
-lbm_status run_block(lbm_ctx* c, int ph, int k) {
+// enqueue n plain steps of a phase as one resident launch
+cudaError_t enqueue_resident(lbm_ctx* c, int ph, int n, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
+    int* err = (int*)(c->sync + 1);
+    const ResPlan& p = c->plan[ph];
+    if (ph == PH_FLOW || ph == PH_ADJ) {
+        FlowLaunch a = flow_base(c);
+        a.fin = c->f[c->fcur];
+        a.fout = c->f[1 - c->fcur];
+        a.ain = c->fa[c->facur];
+        a.aout = c->fa[1 - c->facur];
+        const ResPhase rp = ph == PH_FLOW ? RP_FLOW : (c->thermal ? RP_ADJ_T : RP_ADJ);
+        e = resident_flow(c->stencil, c->storage, rp, a, p, c->inbox, c->sync, err, n, s);
+        (ph == PH_FLOW ? c->fcur : c->facur) ^= 1;
+    } else {
+        ThermLaunch a = therm_base(c);
+        a.gin = c->g[c->gcur];
+        a.gout = c->g[1 - c->gcur];
+        a.ain = c->ga[c->gacur];
+        a.aout = c->ga[1 - c->gacur];
+        e = resident_thermal(c->storage, ph == PH_THERM ? RP_THERM : RP_TADJ, a, p, c->inbox, c->sync, err, n, s);
+        (ph == PH_THERM ? c->gcur : c->gacur) ^= 1;
+    }
+    return e;
+}
+
+// enqueue a block of k steps ending with a reduction, the finalize kernel and
+// the copy of the sums to c->hres
+cudaError_t enqueue_block(lbm_ctx* c, int ph, int k, bool resident, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
+    if (resident)
+        e = enqueue_resident(c, ph, k - 1, s);
+    else
+        for (int i = 0; i < k - 1 && e == cudaSuccess; ++i) e = enqueue_step(c, ph, false, s);
+    if (e == cudaSuccess) e = enqueue_step(c, ph, true, s, resident);
+    if (e != cudaSuccess) return e;
+    e = finalize_launch(c->partials, c->geom.nblocks, phase_nv(ph), c->dres, s, resident ? c->sync : nullptr, k);
+    if (e != cudaSuccess) return e;
+    return cudaMemcpyAsync(c->hres, c->dres, sizeof(double) * (resident ? 3 : phase_nv(ph)), cudaMemcpyDeviceToHost, s);
+}
+
+// One resident launch at a time per device: its blocks wait for one another,
+// so two of them, each partly resident, could wait for ever.  Whoever does not
+// get the gate runs a launch per step (same results) meanwhile.
+std::mutex g_resident_gate[64];
+
+// step numbers are 32 bits: start again from cleared inboxes before they run out
+lbm_status resident_tags(lbm_ctx* c, int k) {
+    c->tags += (unsigned)k;
+    if (c->tags > 0xF0000000ull) {
+        CUDA_TRY(cudaMemsetAsync(c->inbox, 0, c->inbox_bytes, c->stream));
+        CUDA_TRY(cudaMemsetAsync(c->sync, 0, 2 * sizeof(unsigned), c->stream));
+        c->tags = (unsigned)k;
+    }
+    return LBM_OK;
+}
+
+lbm_status run_block(lbm_ctx* c, int ph, int k, bool resident) {
     int& par = parity_of(c, ph);
-    auto key = std::make_tuple(ph, k, par);
+    auto key = std::make_tuple(ph, k, par, resident);
     auto it = c->graphs.find(key);
     if (it == c->graphs.end()) {
         int par0 = par;
         cudaGraph_t graph = nullptr;
         CUDA_TRY(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
-        cudaError_t e = enqueue_block(c, ph, k, c->stream);
+        cudaError_t e = enqueue_block(c, ph, k, resident, c->stream);
         cudaError_t e2 = cudaStreamEndCapture(c->stream, &graph);
         par = par0;  // capture only recorded the work
         if (e != cudaSuccess || e2 != cudaSuccess) {
@@ -277,8 +361,33 @@ lbm_status run_block(lbm_ctx* c, int ph, int k) {
         if (e3 != cudaSuccess) return fail(LBM_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e3));
         it = c->graphs.emplace(key, exec).first;
     }
+    if (resident) {
+        lbm_status st = resident_tags(c, k);
+        if (st != LBM_OK) return st;
+    }
     CUDA_TRY(cudaGraphLaunch(it->second, c->stream));
-    if (k % 2) par ^= 1;
+    // a launch swaps the buffers: once per step, once per resident launch
+    if (!resident && k % 2) par ^= 1;
+    return LBM_OK;
+}
+
+// run a block and wait for it; the sums are in c->hres
+lbm_status run_block_sync(lbm_ctx* c, int ph, int k) {
+    if (resident_fits(c, ph, k - 1)) {
+        std::unique_lock<std::mutex> gate(g_resident_gate[c->device & 63], std::try_to_lock);
+        if (gate.owns_lock()) {
+            lbm_status st = run_block(c, ph, k, true);
+            if (st != LBM_OK) return st;
+            CUDA_TRY(cudaStreamSynchronize(c->stream));
+            if (c->hres[2] == 0.0) return LBM_OK;
+            // a wait gave up: the block's input is untouched and its reducing
+            // step was left out, so the block runs again, a launch per step
+            c->resident = false;
+        }
+    }
+    lbm_status st = run_block(c, ph, k, false);
+    if (st != LBM_OK) return st;
+    CUDA_TRY(cudaStreamSynchronize(c->stream));
     return LBM_OK;
 }
 
@@ -310,9 +419,8 @@ lbm_status run_phase(lbm_ctx* c, int ph, const lbm_solve_opts* o, long long* ste
     double cur = prev;
     while (steps < o->max_steps) {
         long long k = std::min<long long>(K, o->max_steps - steps);
-        lbm_status st = run_block(c, ph, (int)k);
+        lbm_status st = run_block_sync(c, ph, (int)k);
         if (st != LBM_OK) return st;
-        CUDA_TRY(cudaStreamSynchronize(c->stream));
         steps += k;
         double denom = (double)(c->n_nw > 0 ? c->n_nw : 1);
         cur = c->hres[0] / denom;
@@ -574,7 +682,7 @@ lbm_status lbm_check_addressing(int stencil, int nx, int ny, int nz, long long* 
     if (stencil < 0 || stencil > 2) return fail(LBM_ERR_ARG, "unknown stencil");
     if (nx <= 0 || ny <= 0 || nz <= 0) return fail(LBM_ERR_ARG, "lattice sizes must be positive");
     if ((long long)nx * ny * nz > (1LL << 24)) return fail(LBM_ERR_ARG, "at most 2^24 nodes (a host loop)");
-    *mismatches = addressing_mismatches(stencil, nx, ny, nz);
+    *mismatches = addressing_mismatches(stencil, nx, ny, nz) + resident_mismatches(stencil, nx, ny, nz);
     return LBM_OK;
 }
 
@@ -606,6 +714,7 @@ lbm_status lbm_create(lbm_ctx** out, int stencil, int nx, int ny, int nz, int st
     c->ab = adj_bytes(storage);
     c->rb = aux_bytes(storage);
     c->geom = make_geom(nx, ny, nz);
+    c->inbox_bytes = resident_plans(stencil, nx, ny, nz, storage, c->thermal, c->plan);
     cudaError_t e = cudaSuccess;
     e = cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev, cudaEventDisableTiming);
@@ -637,11 +746,24 @@ lbm_status lbm_create(lbm_ctx** out, int stencil, int nx, int ny, int nz, int st
         c->gcn = dalloc(np * c->rb, &e);
     }
     c->partials = (double*)dalloc(sizeof(double) * 2 * (size_t)c->geom.nblocks, &e);
-    c->dres = (double*)dalloc(sizeof(double) * 4, &e);
+    c->dres = (double*)dalloc(sizeof(double) * 4 + 2 * sizeof(unsigned), &e);
+    if (c->inbox_bytes) c->inbox = dalloc(c->inbox_bytes, &e);
+    if (c->dres) c->sync = (unsigned*)(c->dres + 4);
     if (e == cudaSuccess) e = cudaMallocHost(&c->hres, sizeof(double) * 4);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->flags, 1 /* WALL */, np, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->bc, 0, np * 4 * c->rb, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->gamma, 0, np * c->rb, c->stream);
+    if (e == cudaSuccess && c->inbox_bytes) {
+        e = cudaMemsetAsync(c->inbox, 0, c->inbox_bytes, c->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c->sync, 0, 2 * sizeof(unsigned), c->stream);
+        int sms = 0, coop = 0, smem = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c->device);
+        cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
+        c->resident = coop != 0;
+        for (const ResPlan& p : c->plan)
+            if (p.ok) c->resident &= sms * p.per_sm >= p.g.px * p.g.py * p.g.pz && (size_t)smem >= p.smem;
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
         free_all(c);
@@ -1183,12 +1305,21 @@ lbm_status lbm_time_steps(lbm_ctx* c, int phase, int n, double* ms_per_step) {
     if (phase != PH_FLOW && !c->fwd_done) return fail(LBM_ERR_ORDER, "needs a completed lbm_forward");
     if ((st = enter(c)) != LBM_OK) return st;
     const int m = n + (n & 1);  // an even count keeps the buffer parity
+    std::unique_lock<std::mutex> gate(g_resident_gate[c->device & 63], std::defer_lock);
+    const bool resident = resident_fits(c, phase, m / 2) && gate.try_lock();
     int& par = parity_of(c, phase);
     const int par0 = par;
     cudaGraph_t graph = nullptr;
     CUDA_TRY(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
-    for (int i = 0; i < m && e == cudaSuccess; ++i) e = enqueue_step(c, phase, false, c->stream);
+    if (resident) {
+        for (int i = 0; i < 2 && e == cudaSuccess; ++i) {  // an even count of launches, too
+            e = enqueue_resident(c, phase, m / 2, c->stream);
+            if (e == cudaSuccess) e = finalize_launch(c->partials, 0, 1, c->dres, c->stream, c->sync, m);
+        }
+    } else {
+        for (int i = 0; i < m && e == cudaSuccess; ++i) e = enqueue_step(c, phase, false, c->stream);
+    }
     cudaError_t e2 = cudaStreamEndCapture(c->stream, &graph);
     par = par0;
     if (e != cudaSuccess || e2 != cudaSuccess) {
@@ -1200,6 +1331,7 @@ lbm_status lbm_time_steps(lbm_ctx* c, int phase, int n, double* ms_per_step) {
     e = cudaGraphInstantiate(&exec, graph, 0);
     cudaGraphDestroy(graph);
     CUDA_TRY(e);
+    if (resident && (st = resident_tags(c, 4 * m)) != LBM_OK) return st;
     cudaEvent_t e0, e1;
     CUDA_TRY(cudaEventCreate(&e0));
     CUDA_TRY(cudaEventCreate(&e1));
@@ -1213,6 +1345,15 @@ lbm_status lbm_time_steps(lbm_ctx* c, int phase, int n, double* ms_per_step) {
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     cudaGraphExecDestroy(exec);
+    if (resident) {
+        CUDA_TRY(cudaMemcpyAsync(c->hres, c->dres, sizeof(double) * 3, cudaMemcpyDeviceToHost, c->stream));
+        CUDA_TRY(cudaStreamSynchronize(c->stream));
+        if (c->hres[2] != 0.0) {
+            c->resident = false;
+            (phase == PH_FLOW || phase == PH_THERM ? c->fstate : c->astate) = false;
+            return fail(LBM_ERR_CUDA, "a resident launch gave up waiting");
+        }
+    }
     *ms_per_step = (double)ms / m;
     return leave(c);
 }
@@ -1438,6 +1579,8 @@ size_t lbm_footprint_bytes(int stencil, int nx, int ny, int nz, int storage, int
     if (thermal) bytes += 2 * np * 7 * (hb + ab) + np * rb * (1 + 7 + 3 + 1 + 1);
     Geom g = make_geom(nx, ny, nz);
     bytes += sizeof(double) * 2 * (size_t)g.nblocks + 64;
+    ResPlan plans[4] = {};
+    bytes += resident_plans(stencil, nx, ny, nz, storage, thermal != 0, plans);
     return bytes;
 }
 
@@ -1573,7 +1716,7 @@ lbm_status lbm_batch_step(lbm_batch* b, int* n_active) {
     for (int i = 0; i < b->max_slots; ++i) {
         BatchEntry& en = b->e[i];
         if (!en.used || en.phase == SP_DONE || !en.solo) continue;
-        lbm_status st = run_block(en.ctx, slot_to_ctx_phase(en.phase), b->K);
+        lbm_status st = run_block(en.ctx, slot_to_ctx_phase(en.phase), b->K, false);
         if (st != LBM_OK) return st;
         any_solo = true;
     }
