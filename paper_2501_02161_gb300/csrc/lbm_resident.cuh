@@ -157,15 +157,17 @@ struct ResFlow {
     static __device__ __forceinline__ void aux(const Args& a, long long n, int fl, R (&x)[NAUX]) {
         x[0] = (fl & 7) != WALL ? a.gamma[n] : R(0);
     }
-    template <class Bc>
+    static __device__ __forceinline__ bool special(int fl) { return (fl & 7) != FLUID; }
+    // SPECIAL: the node may be other than fluid
+    template <bool SPECIAL, class Bc>
     static __device__ __forceinline__ void update(const Args& a, int fl, const R (&x)[NAUX], R (&f)[L::Q], Bc bc) {
         const int type = fl & 7;
-        if (type >= VEL) {
+        if (SPECIAL && type >= VEL) {
             const R v[3] = {bc(0), bc(1), bc(2)};
             zou_he<L, true>(f, type, (fl >> 3) & 7, v, a.rho0);
         }
         double acc[2];
-        flow_collide<L, T, TA, R, false>(a, 0, fl, x[0], f, acc);
+        flow_collide<L, T, TA, R, false>(a, 0, SPECIAL ? fl : FLUID, x[0], f, acc);
     }
 };
 
@@ -190,13 +192,15 @@ struct ResAdjoint {
             if constexpr (THERMAL) x[4 + k] = a.cpl[k * a.np + n];
         }
     }
-    template <class Bc>
+    static __device__ __forceinline__ bool special(int fl) { return (fl & 7) != FLUID; }
+    template <bool SPECIAL, class Bc>
     static __device__ __forceinline__ void update(const Args& a, int fl, const R (&x)[NAUX], R (&s)[L::Q], Bc) {
         const int type = fl & 7;
         R v0 = 0, v1 = 0, v2 = 0;
         if constexpr (THERMAL) { v0 = x[4]; v1 = x[5]; v2 = x[6]; }
-        adjoint_collide_values<L, R>(a.omega, a.model, a.src_in, type == VEL, x[0], x[1], x[2], x[3], v0, v1, v2, s);
-        if (type >= VEL) zou_he_adjoint<L, true>(s, type, (fl >> 3) & 7);
+        adjoint_collide_values<L, R>(a.omega, a.model, a.src_in, SPECIAL && type == VEL, x[0], x[1], x[2], x[3], v0, v1,
+                                         v2, s);
+        if (SPECIAL && type >= VEL) zou_he_adjoint<L, true>(s, type, (fl >> 3) & 7);
     }
 };
 
@@ -219,14 +223,15 @@ struct ResHeat {
 #pragma unroll
         for (int k = 0; k < 3; ++k) x[2 + k] = a.u[k * a.np + n];
     }
-    template <class Bc>
+    static __device__ __forceinline__ bool special(int fl) { return (fl & 7) != FLUID; }
+    template <bool SPECIAL, class Bc>
     static __device__ __forceinline__ void update(const Args& a, int fl, const R (&x)[NAUX], R (&g)[7], Bc bc) {
         const int type = fl & 7;
-        if (type != FLUID) {
+        if (SPECIAL && type != FLUID) {
             const R v[4] = {R(0), R(0), R(0), bc(0)};
             thermal_bc<R>(g, fl, v, x[1], x[2], x[3], x[4], a.q);
         }
-        if (type != WALL) {
+        if (!SPECIAL || type != WALL) {
             R tem = 0;
 #pragma unroll
             for (int k = 0; k < 7; ++k) tem = Ex<R>::add(tem, g[k]);
@@ -251,10 +256,11 @@ struct ResHeatAdjoint {
     static __device__ __forceinline__ void aux(const Args& a, long long n, int fl, R (&x)[NAUX]) {
         ResHeat<TA, TA, R>::aux(a, n, fl, x);
     }
-    template <class Bc>
+    static __device__ __forceinline__ bool special(int fl) { return (fl & 7) != FLUID; }
+    template <bool SPECIAL, class Bc>
     static __device__ __forceinline__ void update(const Args& a, int fl, const R (&x)[NAUX], R (&s)[7], Bc) {
         R ckn;
-        thermal_adjoint_update<R>(a.src_q, a.src_T, a.beta, fl, x[0], x[1], x[2], x[3], x[4], s, ckn);
+        thermal_adjoint_update<R>(a.src_q, a.src_T, a.beta, SPECIAL ? fl : FLUID, x[0], x[1], x[2], x[3], x[4], s, ckn);
     }
 };
 
@@ -556,7 +562,7 @@ __device__ __forceinline__ void res_node(const typename P::Args& a, const ResGeo
     if (REFLECTS)
         bounce<L>(f);
     else
-        P::update(a, fl, x, f, [&](int c) { return B.aux[(P::NAUX + c) * g.list + j]; });
+        P::template update<BORDER>(a, fl, x, f, [&](int c) { return B.aux[(P::NAUX + c) * g.list + j]; });
     if (last) {
         T* __restrict__ q = P::out(a) + place();
 #pragma unroll
@@ -652,8 +658,9 @@ __global__ void __launch_bounds__(kResThreads(sizeof(typename P::R)), 1)
         sh.own_key[e] = l.own_key;
     }
     __syncthreads();
-    // the three lists.  First every place's list and order in it (open nodes
-    // first, so that they fill warps of their own): 0..2 border, 3 interior, 4
+    // the three lists.  First every place's list and order in it: 0..2 border (the
+    // open nodes first, so that they fill warps of their own; those inside the
+    // box too, so that interior tasks are free of their code), 3 interior, 4
     // wall, 5 not a node.
     unsigned char* const cls = raw + g.word_at;  // the words' list comes here later
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
@@ -670,8 +677,8 @@ __global__ void __launch_bounds__(kResThreads(sizeof(typename P::R)), 1)
             const int fl = a.flags[(b.x0 + lx) + (long long)g.nx * ((b.y0 + ly) + (long long)g.ny * (b.z0 + lz))];
             const int mask = faces(lx, ly, lz);
             if (P::reflects(fl)) c = 4;
-            else if (!mask) c = 3;
-            else c = (fl & 7) >= VEL ? 0 : (mask & 60 ? 1 : 2);
+            else if (P::special(fl)) c = 0;
+            else c = !mask ? 3 : (mask & 60 ? 1 : 2);
         }
         cls[k] = (unsigned char)c;
     }
