@@ -594,16 +594,36 @@ __device__ __forceinline__ void flow_collide(const FlowArgs<T, TA, R>& a, long l
         const R ev = X::fma(-X::mul(R(1.5), k), uu, drho);
         const R k45 = X::mul(R(4.5), k), k3 = X::mul(R(3), k);
         f[0] = X::fma(om1, f[0], X::mul(X::mul(om, R(L::w(0))), ev));
+        // 64-bit arithmetic: one warp's instruction takes 65 cycles here whatever
+        // runs beside it, so the step is its instruction count: the weights of a
+        // direction's class go into the coefficients, three fused operations a
+        // direction instead of four
+        R c45[2], c3[2], c0[2];
+        if constexpr (sizeof(R) == 8) {
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {  // axis, diagonal directions
+                const R omw = X::mul(om, R(L::w(q == 0 ? 1 : L::Q - 1)));
+                c45[q] = X::mul(omw, k45);
+                c3[q] = X::mul(omw, k3);
+                c0[q] = X::mul(omw, ev);
+            }
+        }
 #pragma unroll
         for (int i = 1; i < L::Q; ++i) {
             if (L::opp(i) < i) continue;
             const int j = L::opp(i);
-            const R omw = X::mul(om, R(L::w(i)));
             const R eu = edot_i<L>(i, a0, a1, a2);
-            const R even = X::mul(omw, X::fma(X::mul(k45, eu), eu, ev));
-            const R odd = X::mul(X::mul(omw, k3), eu);
-            f[i] = X::fma(om1, f[i], X::add(even, odd));
-            f[j] = X::fma(om1, f[j], X::sub(even, odd));
+            if constexpr (sizeof(R) == 8) {
+                const int q = L::w(i) == L::w(1) ? 0 : 1;
+                f[i] = X::fma(om1, f[i], X::fma(X::fma(c45[q], eu, c3[q]), eu, c0[q]));
+                f[j] = X::fma(om1, f[j], X::fma(X::fma(c45[q], eu, -c3[q]), eu, c0[q]));
+            } else {
+                const R omw = X::mul(om, R(L::w(i)));
+                const R even = X::mul(omw, X::fma(X::mul(k45, eu), eu, ev));
+                const R odd = X::mul(X::mul(omw, k3), eu);
+                f[i] = X::fma(om1, f[i], X::add(even, odd));
+                f[j] = X::fma(om1, f[j], X::sub(even, odd));
+            }
         }
         // The collision conserves mass: sum h = drho before and after.  With
         // the weights and products rounded, the updated populations sum to
@@ -775,12 +795,21 @@ __global__ void k_flow_init(FlowArgs<T, TA, R> a, int which) {
 template <class L, typename R>
 struct AdjMoments {
     R A, M0, M1, M2, Q00, Q11, Q22, Q01, Q02, Q12;
+    __device__ __forceinline__ void compute_sums(const R (&s)[L::Q]);
     // a direction and its opposite enter A and Q through their sum and M
     // through their difference (e_opp = -e), so each pair is read once
     __device__ __forceinline__ void compute(const R (&s)[L::Q]) {
         using X = Ex<R>;
         M0 = M1 = M2 = Q00 = Q11 = Q22 = Q01 = Q02 = Q12 = R(0);
         A = X::mul(R(L::w(0)), s[0]);
+        if constexpr (sizeof(R) == 8) {  // the weights once per sum (see flow_collide on 64-bit arithmetic)
+            compute_sums(s);
+        } else {
+            compute_pairs(s);
+        }
+    }
+    __device__ __forceinline__ void compute_pairs(const R (&s)[L::Q]) {
+        using X = Ex<R>;
 #pragma unroll
         for (int i = 1; i < L::Q; ++i) {
             if (L::opp(i) < i) continue;
@@ -798,6 +827,63 @@ struct AdjMoments {
         }
     }
 };
+
+// plain sums over the axis pairs and the diagonal pairs of directions, each
+// weighted at its end
+template <class L, typename R>
+__device__ __forceinline__ void AdjMoments<L, R>::compute_sums(const R (&s)[L::Q]) {
+    using X = Ex<R>;
+    R m[3] = {0, 0, 0}, q[3] = {0, 0, 0}, o[3] = {0, 0, 0}, sa = 0, sd = 0, am[3] = {0, 0, 0}, aq[3] = {0, 0, 0};
+    bool any_a = false, any_d = false, any_c[3] = {false, false, false}, any_o[3] = {false, false, false};
+#pragma unroll
+    for (int i = 1; i < L::Q; ++i) {
+        if (L::opp(i) < i) continue;
+        const int j = L::opp(i);
+        const R p = X::add(s[i], s[j]), d = X::sub(s[i], s[j]);
+        const int e[3] = {L::cx(i), L::cy(i), L::cz(i)};
+        if (L::w(i) == L::w(1)) {
+            sa = any_a ? X::add(sa, p) : p;
+            any_a = true;
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+                if (e[a]) {
+                    am[a] = e[a] > 0 ? d : -d;
+                    aq[a] = p;
+                }
+            continue;
+        }
+        sd = any_d ? X::add(sd, p) : p;
+        any_d = true;
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            if (e[a]) {
+                m[a] = any_c[a] ? add_s(m[a], e[a], d) : (e[a] > 0 ? d : -d);
+                q[a] = any_c[a] ? X::add(q[a], p) : p;
+                any_c[a] = true;
+            }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {  // xy, xz, yz
+            const int x = e[a == 2 ? 1 : 0] * e[a == 0 ? 1 : 2];
+            if (x) {
+                o[a] = any_o[a] ? add_s(o[a], x, p) : (x > 0 ? p : -p);
+                any_o[a] = true;
+            }
+        }
+    }
+    const R wa = R(L::w(1)), wd = R(L::w(L::Q - 1));
+    A = X::fma(wd, sd, X::fma(wa, sa, A));
+    M0 = X::fma(wa, am[0], X::mul(wd, m[0]));
+    M1 = X::fma(wa, am[1], X::mul(wd, m[1]));
+    Q00 = X::fma(wa, aq[0], X::mul(wd, q[0]));
+    Q11 = X::fma(wa, aq[1], X::mul(wd, q[1]));
+    Q01 = X::mul(wd, o[0]);
+    if constexpr (L::D == 3) {
+        M2 = X::fma(wa, am[2], X::mul(wd, m[2]));
+        Q22 = X::fma(wa, aq[2], X::mul(wd, q[2]));
+        Q02 = X::mul(wd, o[1]);
+        Q12 = X::mul(wd, o[2]);
+    }
+}
 
 template <class L, bool MIRROR, typename T, typename TA, typename R>
 __device__ __forceinline__ void pull_adjoint(const FlowArgs<T, TA, R>& a, const Cell& c, R (&s)[L::Q]) {
