@@ -243,6 +243,24 @@ __device__ __forceinline__ Cell this_cell(int nx, int ny) {
     return c;
 }
 
+// the node of a thread of a plain step over widths off a multiple of 32: 256
+// consecutive nodes a block.  A row then starts anywhere in a 128-byte line;
+// tiles cut such lines between warps and leave lanes idle at every row's end.
+// 147 x 140 x 130: forward 76.4 -> 63.7 us, adjoint 76.5 -> 70.6; 129 x 96 x 80
+// coupled adjoint 37.7 -> 30.9.  Multiples of 32 keep the tiles (the divisions
+// cost the adjoint 2 % there).
+__device__ __forceinline__ Cell linear_cell(int nx, int ny, int nz) {
+    const unsigned n = blockIdx.x * blockDim.x + threadIdx.x;  // below 2^31
+    const unsigned row = n / (unsigned)nx;
+    Cell c;
+    c.x = (int)(n - row * (unsigned)nx);
+    c.z = (int)(row / (unsigned)ny);
+    c.y = (int)(row - (unsigned)c.z * (unsigned)ny);
+    c.n = n;
+    c.active = c.z < nz;
+    return c;
+}
+
 // offsets (in nodes) from a node to its six axis neighbours, periodic wrap
 // included; they fit in 32 bits because node counts stay below 2^31.  A pull
 // then costs one integer add per population instead of a wrapped 3-D index.
@@ -667,12 +685,12 @@ struct FwdMinBlocks {
 };
 
 // bail (or null): a reducing step that finds the flag set leaves everything as it is
-template <class L, typename T, typename TA, typename R, bool REDUCE, bool MIRROR>
+template <class L, typename T, typename TA, typename R, bool REDUCE, bool MIRROR, bool LINEAR = false>
 __global__ void __launch_bounds__(256, (FwdMinBlocks<L, T>::value)) k_flow_step(FlowArgs<T, TA, R> a, const int* bail) {
     pdl_launch_dependents();
     pdl_wait();
     if (REDUCE && bail && *bail) return;
-    const Cell c = this_cell(a.nx, a.ny);
+    const Cell c = LINEAR ? linear_cell(a.nx, a.ny, a.nz) : this_cell(a.nx, a.ny);
     double acc[2] = {0.0, 0.0};
     if (c.active) flow_step_node<L, T, TA, R, REDUCE, MIRROR>(a, c, acc);
     if (REDUCE) block_partials<2>(acc, a.partials, grid_block_id());
@@ -902,7 +920,8 @@ __device__ __forceinline__ void pull_adjoint(const FlowArgs<T, TA, R>& a, const 
 // resident 256-thread blocks per SM requested from the compiler: the plain
 // FP32-math D3Q19 adjoint fits 40 registers without spilling (6 blocks, 75 %
 // occupancy), its thermal-coupling variant 48 (5 blocks); the reducing
-// variants (one step in K) keep the compiler's choice
+// variants (one step in K) keep the compiler's choice; the plain adjoint over
+// consecutive nodes takes 48 (8 bytes would spill at 40)
 template <class L, typename R, bool REDUCE, bool THERMAL>
 struct AdjMinBlocks {
     static constexpr int value =
@@ -986,13 +1005,13 @@ __device__ __forceinline__ void flow_adjoint_node(const FlowArgs<T, TA, R>& a, c
     }
 }
 
-template <class L, typename T, typename TA, typename R, bool REDUCE, bool THERMAL, bool MIRROR>
-__global__ void __launch_bounds__(256, (AdjMinBlocks<L, R, REDUCE, THERMAL>::value))
+template <class L, typename T, typename TA, typename R, bool REDUCE, bool THERMAL, bool MIRROR, bool LINEAR = false>
+__global__ void __launch_bounds__(256, (AdjMinBlocks<L, R, REDUCE, THERMAL || LINEAR>::value))
     k_flow_adjoint(FlowArgs<T, TA, R> a, const int* bail) {
     pdl_launch_dependents();
     pdl_wait();
     if (REDUCE && bail && *bail) return;
-    const Cell c = this_cell(a.nx, a.ny);
+    const Cell c = LINEAR ? linear_cell(a.nx, a.ny, a.nz) : this_cell(a.nx, a.ny);
     double acc[1] = {0.0};
     if (c.active) flow_adjoint_node<L, T, TA, R, REDUCE, THERMAL, false, MIRROR>(a, c, acc);
     if (REDUCE) block_partials<1>(acc, a.partials, grid_block_id());
@@ -1279,12 +1298,12 @@ __global__ void __launch_bounds__(256) k_thermal_collide_initial(ThermArgs<T, TA
         Pop<T>::st(a.gout, (size_t)k * a.np + c.n, g[k], R(D3Q7::w(k)) * a.T0);
 }
 
-template <typename T, typename TA, typename R, bool REDUCE, bool MIRROR>
+template <typename T, typename TA, typename R, bool REDUCE, bool MIRROR, bool LINEAR = false>
 __global__ void __launch_bounds__(256) k_thermal_step(ThermArgs<T, TA, R> a, const int* bail) {
     pdl_launch_dependents();
     pdl_wait();
     if (REDUCE && bail && *bail) return;
-    const Cell c = this_cell(a.nx, a.ny);
+    const Cell c = LINEAR ? linear_cell(a.nx, a.ny, a.nz) : this_cell(a.nx, a.ny);
     double acc[2] = {0.0, 0.0};
     if (c.active) thermal_step_node<T, TA, R, REDUCE, MIRROR>(a, c, acc);
     if (REDUCE) block_partials<2>(acc, a.partials, grid_block_id());
@@ -1403,12 +1422,12 @@ __device__ __forceinline__ void thermal_adjoint_node(const ThermArgs<T, TA, R>& 
     }
 }
 
-template <typename T, typename TA, typename R, bool REDUCE, bool MIRROR>
+template <typename T, typename TA, typename R, bool REDUCE, bool MIRROR, bool LINEAR = false>
 __global__ void __launch_bounds__(256) k_thermal_adjoint(ThermArgs<T, TA, R> a, const int* bail) {
     pdl_launch_dependents();
     pdl_wait();
     if (REDUCE && bail && *bail) return;
-    const Cell c = this_cell(a.nx, a.ny);
+    const Cell c = LINEAR ? linear_cell(a.nx, a.ny, a.nz) : this_cell(a.nx, a.ny);
     double acc[1] = {0.0};
     if (c.active) thermal_adjoint_node<T, TA, R, REDUCE, MIRROR>(a, c, acc);
     if (REDUCE) block_partials<1>(acc, a.partials, grid_block_id());

@@ -117,6 +117,7 @@ void flow_dispatch_m(FlowOp op, const FlowLaunch& l, const Geom& g, cudaStream_t
     using TA = typename StorageTypes<S>::TA;
     using R = typename StorageTypes<S>::R;
     auto a = flow_args<S>(l);
+    const bool linear = g.linear;
     switch (op) {
         case FOP_INIT_F: k_flow_init<L, T, TA, R><<<flat_grid(l.np), 256, 0, s>>>(a, 0); break;
         case FOP_INIT_A: k_flow_init<L, T, TA, R><<<flat_grid(l.np), 256, 0, s>>>(a, 1); break;
@@ -130,12 +131,25 @@ void flow_dispatch_m(FlowOp op, const FlowLaunch& l, const Geom& g, cudaStream_t
                     break;
                 }
             }
-            launch_pdl(k_flow_step<L, T, TA, R, false, M>, g, s, a, l.bail);
+            if (linear)
+                launch_pdl(k_flow_step<L, T, TA, R, false, M, true>, g, s, a, l.bail);
+            else
+                launch_pdl(k_flow_step<L, T, TA, R, false, M>, g, s, a, l.bail);
             break;
         case FOP_STEP_RED: launch_pdl(k_flow_step<L, T, TA, R, true, M>, g, s, a, l.bail); break;
-        case FOP_ADJ: launch_pdl(k_flow_adjoint<L, T, TA, R, false, false, M>, g, s, a, l.bail); break;
+        case FOP_ADJ:
+            if (linear)
+                launch_pdl(k_flow_adjoint<L, T, TA, R, false, false, M, true>, g, s, a, l.bail);
+            else
+                launch_pdl(k_flow_adjoint<L, T, TA, R, false, false, M>, g, s, a, l.bail);
+            break;
         case FOP_ADJ_RED: launch_pdl(k_flow_adjoint<L, T, TA, R, true, false, M>, g, s, a, l.bail); break;
-        case FOP_ADJ_T: launch_pdl(k_flow_adjoint<L, T, TA, R, false, true, M>, g, s, a, l.bail); break;
+        case FOP_ADJ_T:
+            if (linear)
+                launch_pdl(k_flow_adjoint<L, T, TA, R, false, true, M, true>, g, s, a, l.bail);
+            else
+                launch_pdl(k_flow_adjoint<L, T, TA, R, false, true, M>, g, s, a, l.bail);
+            break;
         case FOP_ADJ_T_RED: launch_pdl(k_flow_adjoint<L, T, TA, R, true, true, M>, g, s, a, l.bail); break;
         case FOP_SENS: k_flow_sens<L, T, TA, R, false, M><<<g.grid, g.block, 0, s>>>(a); break;
         case FOP_SENS_T: k_flow_sens<L, T, TA, R, true, M><<<g.grid, g.block, 0, s>>>(a); break;
@@ -170,12 +184,23 @@ void therm_dispatch_m(ThermOp op, const ThermLaunch& l, const Geom& g, cudaStrea
     using TA = typename StorageTypes<S>::TA;
     using R = typename StorageTypes<S>::R;
     auto a = therm_args<S>(l);
+    const bool linear = g.linear;
     switch (op) {
         case TOP_INIT_G: k_thermal_init<T, TA, R><<<flat_grid(l.np), 256, 0, s>>>(a, 0); break;
         case TOP_INIT_A: k_thermal_init<T, TA, R><<<flat_grid(l.np), 256, 0, s>>>(a, 1); break;
-        case TOP_STEP: launch_pdl(k_thermal_step<T, TA, R, false, M>, g, s, a, l.bail); break;
+        case TOP_STEP:
+            if (linear)
+                launch_pdl(k_thermal_step<T, TA, R, false, M, true>, g, s, a, l.bail);
+            else
+                launch_pdl(k_thermal_step<T, TA, R, false, M>, g, s, a, l.bail);
+            break;
         case TOP_STEP_RED: launch_pdl(k_thermal_step<T, TA, R, true, M>, g, s, a, l.bail); break;
-        case TOP_ADJ: launch_pdl(k_thermal_adjoint<T, TA, R, false, M>, g, s, a, l.bail); break;
+        case TOP_ADJ:
+            if (linear)
+                launch_pdl(k_thermal_adjoint<T, TA, R, false, M, true>, g, s, a, l.bail);
+            else
+                launch_pdl(k_thermal_adjoint<T, TA, R, false, M>, g, s, a, l.bail);
+            break;
         case TOP_ADJ_RED: launch_pdl(k_thermal_adjoint<T, TA, R, true, M>, g, s, a, l.bail); break;
         case TOP_COUPLING: k_thermal_coupling<T, TA, R, M><<<g.grid, g.block, 0, s>>>(a); break;
         case TOP_COLLIDE_INIT: k_thermal_collide_initial<T, TA, R><<<g.grid, g.block, 0, s>>>(a); break;

@@ -11,12 +11,16 @@ struct Geom {
     dim3 grid;
     dim3 block;
     long long nblocks;  // grid.x * grid.y * grid.z (reduction partial count)
+    bool linear;        // blocks of consecutive nodes instead of tiles (make_step_geom)
 };
 
 // (BX x BY) tiles of x-y planes, one thread per node, `threads` per block
 // when the lattice is wide enough; BX divides nx when possible so no lane
 // idles.
 Geom make_geom(int nx, int ny, int nz, int threads = 256);
+// the same for a step that sums nothing: blocks of consecutive nodes where rows
+// are no multiple of 32
+Geom make_step_geom(int nx, int ny, int nz);
 
 struct FlowLaunch {
     const void* fin;

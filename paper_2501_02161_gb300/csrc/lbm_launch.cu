@@ -17,6 +17,17 @@ Geom make_geom(int nx, int ny, int nz, int threads) {
     g.block = dim3(bx, by, 1);
     g.grid = dim3((nx + bx - 1) / bx, (ny + by - 1) / by, nz);
     g.nblocks = (long long)g.grid.x * g.grid.y * g.grid.z;
+    g.linear = false;
+    return g;
+}
+
+Geom make_step_geom(int nx, int ny, int nz) {
+    if (nx % 32 == 0) return make_geom(nx, ny, nz);
+    Geom g;
+    g.block = dim3(256, 1, 1);
+    g.grid = dim3((unsigned)(((long long)nx * ny * nz + 255) / 256), 1, 1);
+    g.nblocks = g.grid.x;
+    g.linear = true;
     return g;
 }
 

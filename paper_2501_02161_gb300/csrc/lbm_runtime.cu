@@ -95,6 +95,7 @@ struct lbm_ctx {
     bool resident = false;
 
     Geom geom{};
+    Geom step_geom{};  // of the plain steps
     lbm_params prm{0.6, 1.0, 0, 0.0, 1.0, 0.0, 0.0, 0.0};
     lbm_objective obj{1.0, 0.0, 0.0};
     long long n_in = 0, n_nw = 0;
@@ -230,6 +231,8 @@ int phase_nv(int ph) { return ph == PH_FLOW || ph == PH_THERM ? 2 : 1; }
 cudaError_t enqueue_step(lbm_ctx* c, int ph, bool reduce, cudaStream_t s, bool after_resident = false) {
     cudaError_t e = cudaSuccess;
     const int* bail = after_resident ? (const int*)(c->sync + 1) : nullptr;
+    const bool cont = ph == PH_ADJ && c->adj_scheme == LBM_ADJOINT_CONTINUOUS;  // keeps the tiles
+    const Geom& geom = reduce || cont ? c->geom : c->step_geom;
     if (ph == PH_FLOW) {
         FlowLaunch a = flow_base(c);
         a.fin = c->f[c->fcur];
@@ -237,7 +240,7 @@ cudaError_t enqueue_step(lbm_ctx* c, int ph, bool reduce, cudaStream_t s, bool a
         a.out0 = c->rho;
         a.out1 = c->u;
         a.bail = bail;
-        e = flow_launch(c->stencil, c->storage, reduce ? FOP_STEP_RED : FOP_STEP, a, c->geom, s);
+        e = flow_launch(c->stencil, c->storage, reduce ? FOP_STEP_RED : FOP_STEP, a, geom, s);
         c->fcur ^= 1;
     } else if (ph == PH_THERM) {
         ThermLaunch a = therm_base(c);
@@ -246,7 +249,7 @@ cudaError_t enqueue_step(lbm_ctx* c, int ph, bool reduce, cudaStream_t s, bool a
         a.out0 = c->T;
         a.out1 = c->gpost;
         a.bail = bail;
-        e = thermal_launch(c->storage, reduce ? TOP_STEP_RED : TOP_STEP, a, c->geom, s);
+        e = thermal_launch(c->storage, reduce ? TOP_STEP_RED : TOP_STEP, a, geom, s);
         c->gcur ^= 1;
     } else if (ph == PH_ADJ) {
         FlowLaunch a = flow_base(c);
@@ -255,14 +258,14 @@ cudaError_t enqueue_step(lbm_ctx* c, int ph, bool reduce, cudaStream_t s, bool a
         a.bail = bail;
         FlowOp op = c->thermal ? (reduce ? FOP_ADJ_T_RED : FOP_ADJ_T) : (reduce ? FOP_ADJ_RED : FOP_ADJ);
         if (c->adj_scheme == LBM_ADJOINT_CONTINUOUS) op = reduce ? FOP_ADJ_CONT_RED : FOP_ADJ_CONT;
-        e = flow_launch(c->stencil, c->storage, op, a, c->geom, s);
+        e = flow_launch(c->stencil, c->storage, op, a, geom, s);
         c->facur ^= 1;
     } else {
         ThermLaunch a = therm_base(c);
         a.ain = c->ga[c->gacur];
         a.aout = c->ga[1 - c->gacur];
         a.bail = bail;
-        e = thermal_launch(c->storage, reduce ? TOP_ADJ_RED : TOP_ADJ, a, c->geom, s);
+        e = thermal_launch(c->storage, reduce ? TOP_ADJ_RED : TOP_ADJ, a, geom, s);
         c->gacur ^= 1;
     }
     return e;
@@ -714,6 +717,7 @@ lbm_status lbm_create(lbm_ctx** out, int stencil, int nx, int ny, int nz, int st
     c->ab = adj_bytes(storage);
     c->rb = aux_bytes(storage);
     c->geom = make_geom(nx, ny, nz);
+    c->step_geom = make_step_geom(nx, ny, nz);
     c->inbox_bytes = resident_plans(stencil, nx, ny, nz, storage, c->thermal, c->plan);
     cudaError_t e = cudaSuccess;
     e = cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking);
