@@ -303,6 +303,12 @@ lbm_status lbm_get_adjoint(lbm_ctx* ctx, void* fstar, void* gstar, int dtype, in
  * phases 1-3, a completed lbm_forward. */
 lbm_status lbm_time_steps(lbm_ctx* ctx, int phase, int n, double* ms_per_step);
 
+/* Kernels that the context's initialisations, solves and sensitivities have
+ * launched since it was created (0 for null): a block of k steps is k + 1 of
+ * them, or 3 when its plain steps are one resident launch.  Type conversions of
+ * inputs and outputs, lbm_time_steps and packed batch launches are not counted. */
+long long lbm_launches(lbm_ctx* ctx);
+
 /* ---------------------------------------------------------------------------
  * Checkpoint / resume of a context's solver state (no counterpart in the
  * paper).  The state is the current forward and adjoint populations (and the

@@ -44,14 +44,14 @@
 //
 // The node arithmetic is that of the one-step kernels, operation by operation.
 //
-// Measured, us a step against one launch per step (forward / adjoint): 16^3
-// 1.83 / 1.80 against 2.27 / 2.56, 32^3 2.5 against 3.1 / 2.8, 64^3 FP32 5.0 /
-// 4.9 against 5.65 / 5.73 (4.7 in blocks of 500 steps: the set-up of a launch
-// is about 25 us), temperature at 192 x 48 x 24 2.26 / 2.02 against 3.29 / 3.46,
-// FP64 at 16^3 8.8 / 7.8 against 23.9 / 27.2.  At 64^3 a block issues 18300 warp
-// instructions a step (4600 cycles of each scheduler) and takes 10000 cycles:
-// what bounds it is the chain border - barrier - words - barrier, of which the
-// travel of the words is about 1500.
+// Measured, us a step (forward / adjoint) in launches of 500 steps against one
+// launch per step: 16^3 1.76 / 1.63 against 2.27 / 2.56, 32^3 2.23 / 2.22 against
+// 3.1 / 2.8, 64^3 FP32 4.38 / 4.33 against 5.65 / 5.73, temperature at
+// 192 x 48 x 24 1.84 / 1.76 against 3.29 / 3.46; 32^3 FP64, 300 steps of each,
+// 9.8 against 18.5 ms.  The set-up of a launch is about 25 us.  At 64^3 a block
+// issues 18300 warp instructions a step (4600 cycles of each scheduler) and takes
+// about 8500 cycles: what bounds it is the chain border - barrier - words -
+// barrier, of which the travel of the words is about 1500.
 #pragma once
 
 #include "lbm_device.cuh"
@@ -196,10 +196,8 @@ struct ResAdjoint {
     template <bool SPECIAL, class Bc>
     static __device__ __forceinline__ void update(const Args& a, int fl, const R (&x)[NAUX], R (&s)[L::Q], Bc) {
         const int type = fl & 7;
-        R v0 = 0, v1 = 0, v2 = 0;
-        if constexpr (THERMAL) { v0 = x[4]; v1 = x[5]; v2 = x[6]; }
-        adjoint_collide_values<L, R>(a.omega, a.model, a.src_in, SPECIAL && type == VEL, x[0], x[1], x[2], x[3], v0, v1,
-                                         v2, s);
+        adjoint_collide_values<L, R>(
+            a, SPECIAL && type == VEL, [&](int c) -> R { return c < NAUX ? x[c < NAUX ? c : 0] : R(0); }, s);
         if (SPECIAL && type >= VEL) zou_he_adjoint<L, true>(s, type, (fl >> 3) & 7);
     }
 };

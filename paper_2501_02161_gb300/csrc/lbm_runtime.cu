@@ -93,6 +93,7 @@ struct lbm_ctx {
     size_t inbox_bytes = 0;
     unsigned long long tags = 0;  // step numbers used since the counter was cleared
     bool resident = false;
+    long long launches = 0;  // kernels launched (lbm_launches)
 
     Geom geom{};
     Geom step_geom{};  // of the plain steps
@@ -369,6 +370,7 @@ lbm_status run_block(lbm_ctx* c, int ph, int k, bool resident) {
         if (st != LBM_OK) return st;
     }
     CUDA_TRY(cudaGraphLaunch(it->second, c->stream));
+    c->launches += resident ? 3 : k + 1;  // steps, reducing step, finalize
     // a launch swaps the buffers: once per step, once per resident launch
     if (!resident && k % 2) par ^= 1;
     return LBM_OK;
@@ -379,12 +381,15 @@ lbm_status run_block_sync(lbm_ctx* c, int ph, int k) {
     if (resident_fits(c, ph, k - 1)) {
         std::unique_lock<std::mutex> gate(g_resident_gate[c->device & 63], std::try_to_lock);
         if (gate.owns_lock()) {
-            lbm_status st = run_block(c, ph, k, true);
-            if (st != LBM_OK) return st;
-            CUDA_TRY(cudaStreamSynchronize(c->stream));
-            if (c->hres[2] == 0.0) return LBM_OK;
-            // a wait gave up: the block's input is untouched and its reducing
-            // step was left out, so the block runs again, a launch per step
+            if (run_block(c, ph, k, true) == LBM_OK) {
+                CUDA_TRY(cudaStreamSynchronize(c->stream));
+                if (c->hres[2] == 0.0) return LBM_OK;
+            } else {
+                (void)cudaGetLastError();
+            }
+            // the launch was refused, or a wait gave up (the block's input is
+            // untouched and its reducing step was left out): the block runs
+            // again, a launch per step
             c->resident = false;
         }
     }
@@ -528,6 +533,7 @@ lbm_status init_flow(lbm_ctx* c) {
     a.out1 = c->u;
     c->fcur = 0;
     CUDA_TRY(flow_launch(c->stencil, c->storage, FOP_INIT_F, a, c->geom, c->stream));
+    ++c->launches;
     c->last_I[PH_FLOW] = 0.0;
     return LBM_OK;
 }
@@ -539,6 +545,7 @@ lbm_status init_temperature(lbm_ctx* c) {
     t.out1 = c->gpost;
     c->gcur = 0;
     CUDA_TRY(thermal_launch(c->storage, TOP_INIT_G, t, c->geom, c->stream));
+    ++c->launches;
     c->last_I[PH_THERM] = c->prm.T0;
     c->g_fresh = true;
     return LBM_OK;
@@ -551,6 +558,7 @@ lbm_status collide_initial_temperature(lbm_ctx* c) {
     ThermLaunch t = therm_base(c);
     t.gout = c->g[c->gcur];
     CUDA_TRY(thermal_launch(c->storage, TOP_COLLIDE_INIT, t, c->geom, c->stream));
+    ++c->launches;
     c->g_fresh = false;
     return LBM_OK;
 }
@@ -566,6 +574,7 @@ lbm_status init_flow_adjoint(lbm_ctx* c) {
     a.aout = c->fa[0];
     c->facur = 0;
     CUDA_TRY(flow_launch(c->stencil, c->storage, FOP_INIT_A, a, c->geom, c->stream));
+    ++c->launches;
     c->last_I[PH_ADJ] = 0.0;
     return LBM_OK;
 }
@@ -575,6 +584,7 @@ lbm_status init_temperature_adjoint(lbm_ctx* c) {
     t.aout = c->ga[0];
     c->gacur = 0;
     CUDA_TRY(thermal_launch(c->storage, TOP_INIT_A, t, c->geom, c->stream));
+    ++c->launches;
     CUDA_TRY(cudaMemsetAsync(c->cpl, 0, 3 * c->np * c->rb, c->stream));
     CUDA_TRY(cudaMemsetAsync(c->sT, 0, c->np * c->rb, c->stream));
     c->last_I[PH_TADJ] = 0.0;
@@ -596,6 +606,7 @@ lbm_status run_coupling(lbm_ctx* c) {
     t.out0 = c->cpl;
     t.out1 = c->sT;
     CUDA_TRY(thermal_launch(c->storage, TOP_COUPLING, t, c->geom, c->stream));
+    ++c->launches;
     return LBM_OK;
 }
 
@@ -1121,6 +1132,7 @@ lbm_status lbm_sensitivity(lbm_ctx* c, void* out, int dtype, int on_device) {
     a.out0 = c->sens;
     const FlowOp op = c->adj_scheme == LBM_ADJOINT_CONTINUOUS ? FOP_SENS_CONT : (c->thermal ? FOP_SENS_T : FOP_SENS);
     CUDA_TRY(flow_launch(c->stencil, c->storage, op, a, c->geom, c->stream));
+    ++c->launches;
     st = copy_out(c, out, c->sens, 1, dtype, on_device);
     if (st != LBM_OK) return st;
     return leave(c);
@@ -1216,6 +1228,8 @@ size_t state_size(lbm_ctx* c) {
 }  // namespace
 
 extern "C" {
+
+long long lbm_launches(lbm_ctx* c) { return c ? c->launches : 0; }
 
 size_t lbm_state_bytes(lbm_ctx* c) { return c ? state_size(c) : 0; }
 

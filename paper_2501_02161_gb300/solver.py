@@ -255,9 +255,14 @@ class Solver:
         C.check(self.lib.lbm_import_state(self._ctx, ctypes.c_void_p(state.data_ptr()),
                                           state.numel()), "lbm_import_state")
 
+    def launches(self) -> int:
+        """Kernels launched by this context's solves so far."""
+        return int(self.lib.lbm_launches(self._ctx))
+
     def time_steps(self, phase: int, n: int) -> float:
-        """Mean ms per plain fused step of a phase (0 flow, 1 temperature,
-        2 flow adjoint, 3 temperature adjoint), CUDA events on its stream."""
+        """Mean ms per plain step of a phase as a solve runs it (0 flow,
+        1 temperature, 2 flow adjoint, 3 temperature adjoint), CUDA events on
+        its stream."""
         ms = ctypes.c_double()
         self._stream()
         C.check(self.lib.lbm_time_steps(self._ctx, int(phase), int(n), ctypes.byref(ms)),

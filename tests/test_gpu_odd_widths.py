@@ -1,5 +1,5 @@
 """Plain steps over blocks of consecutive nodes (rows off a multiple of 32)
-against the FP64 reference lattice solve and against tiles.
+against tiles of x-y planes.
 
 A block of check_every = 1 runs its one step through the reducing kernel, which
 keeps the tiles; longer ones run their plain steps over consecutive nodes.  Both
