@@ -49,7 +49,7 @@
 // 3.1 / 2.8, 64^3 FP32 4.38 / 4.33 against 5.65 / 5.73, temperature at
 // 192 x 48 x 24 1.84 / 1.76 against 3.29 / 3.46; 32^3 FP64, 300 steps of each,
 // 9.8 against 18.5 ms.  The set-up of a launch is about 25 us.  At 64^3 a block
-// issues 18300 warp instructions a step (4600 cycles of each scheduler) and takes
+// issues 20000 warp instructions a step (5000 cycles of each scheduler) and takes
 // about 8500 cycles: what bounds it is the chain border - barrier - words -
 // barrier, of which the travel of the words is about 1500.
 #pragma once
@@ -196,8 +196,10 @@ struct ResAdjoint {
     template <bool SPECIAL, class Bc>
     static __device__ __forceinline__ void update(const Args& a, int fl, const R (&x)[NAUX], R (&s)[L::Q], Bc) {
         const int type = fl & 7;
-        adjoint_collide_values<L, R>(
-            a, SPECIAL && type == VEL, [&](int c) -> R { return c < NAUX ? x[c < NAUX ? c : 0] : R(0); }, s);
+        R v0 = 0, v1 = 0, v2 = 0;
+        if constexpr (THERMAL) { v0 = x[4]; v1 = x[5]; v2 = x[6]; }
+        adjoint_collide_values<L, R>(a.omega, a.model, a.src_in, SPECIAL && type == VEL, x[0], x[1], x[2], x[3], v0, v1,
+                                         v2, s);
         if (SPECIAL && type >= VEL) zou_he_adjoint<L, true>(s, type, (fl >> 3) & 7);
     }
 };
