@@ -309,6 +309,15 @@ lbm_status lbm_time_steps(lbm_ctx* ctx, int phase, int n, double* ms_per_step);
  * inputs and outputs, lbm_time_steps and packed batch launches are not counted. */
 long long lbm_launches(lbm_ctx* ctx);
 
+/* How the context's resident launches wait and count (no effect on a lattice
+ * that has none): wait_limit, the polls after which a wait gives up and the
+ * steps run again a launch each (by default 2^21, about a second; 0: a word
+ * that is not there at the first poll is given up), and step_number, from which
+ * the steps are numbered on (they start again from 0 before 2^32).  For tests
+ * of what a waiting block and a long run do: ordinary programs have no use for
+ * it.  Errors: LBM_ERR_ARG (null, wait_limit < 0). */
+lbm_status lbm_set_resident(lbm_ctx* ctx, int wait_limit, unsigned step_number);
+
 /* ---------------------------------------------------------------------------
  * Checkpoint / resume of a context's solver state (no counterpart in the
  * paper).  The state is the current forward and adjoint populations (and the

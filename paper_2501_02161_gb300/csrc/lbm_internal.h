@@ -112,13 +112,20 @@ enum ResPhase { RP_FLOW = 0, RP_THERM, RP_ADJ, RP_TADJ, RP_ADJ_T };
 // cut of a lattice for a phase (ok = false: it does not fit on the chip); a
 // function of the sizes alone, for the 152 SMs of a GB300
 ResPlan resident_plan(int stencil, int storage, ResPhase ph, int nx, int ny, int nz);
+constexpr int kWaitLimit = 1 << 21;  // polls of about 0.5 us: about a second
+// the words that the boxes exchange
+struct ResWords {
+    void* inboxes;
+    const unsigned* base;  // the steps of the words are numbered from here
+    int* err;              // set when a wait gave up
+    int limit;             // polls after which it does
+};
 // `steps` plain steps of a phase in one cooperative launch: reads fin / ain /
-// gin, writes fout / aout / gout.  base: step numbers of the words start here;
-// err is set when a wait gave up.
-cudaError_t resident_flow(int stencil, int storage, ResPhase ph, const FlowLaunch& a, const ResPlan& p, void* inboxes,
-                          const unsigned* base, int* err, int steps, cudaStream_t s);
-cudaError_t resident_thermal(int storage, ResPhase ph, const ThermLaunch& a, const ResPlan& p, void* inboxes,
-                             const unsigned* base, int* err, int steps, cudaStream_t s);
+// gin, writes fout / aout / gout
+cudaError_t resident_flow(int stencil, int storage, ResPhase ph, const FlowLaunch& a, const ResPlan& p,
+                          const ResWords& w, int steps, cudaStream_t s);
+cudaError_t resident_thermal(int storage, ResPhase ph, const ThermLaunch& a, const ResPlan& p, const ResWords& w,
+                             int steps, cudaStream_t s);
 
 // storage codes follow lbm_storage; stencil codes follow lbm_stencil
 cudaError_t flow_launch(int stencil, int storage, FlowOp op, const FlowLaunch& a, const Geom& g,

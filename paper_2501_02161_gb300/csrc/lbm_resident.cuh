@@ -39,7 +39,7 @@
 // wall node reflects every population: value opp(i) becomes value i, which is
 // the slot's content already, so walls take no part in the steps.
 //
-// Every wait is bounded: after kSpinLimit polls the block sets an error flag,
+// Every wait is bounded: after kWaitLimit polls the block sets an error flag,
 // waits no more and the launch ends; the input populations are untouched.
 //
 // The node arithmetic is that of the one-step kernels, operation by operation.
@@ -58,8 +58,6 @@
 #include "lbm_internal.h"
 
 namespace lbm {
-
-constexpr int kSpinLimit = 1 << 21;  // polls of about 0.5 us: about a second
 
 // ---------------------------------------------------------------------------
 // one exchanged word: values and step number, written and read whole
@@ -291,6 +289,7 @@ struct ResShared {
     int lane[3][32];        // nodes of a list and lane
     int over[3];            // nodes placed beyond their lane's share
     int bail;
+    int limit;              // polls of a wait
 };
 static_assert(sizeof(ResShared) <= kResHead, "head of the shared memory");
 
@@ -474,8 +473,11 @@ __device__ __forceinline__ void res_receive(const ResBlock<P>& B, const ResGeom&
             for (int u = 0; u < U; ++u) v[u] = word_ld(own + (t + u * nt < g.inbox ? t + u * nt : t));
 #pragma unroll
             for (int u = 0; u < U; ++u) bad |= word_tag(v[u]) ^ tag;
-            if (!__any_sync(0xffffffffu, bad) || *(volatile int*)&B.sh->bail) break;
-            if (spins > kSpinLimit) {
+            // both are decisions of the whole warp: a lane that left by itself
+            // would be missing in the others' next vote
+            if (!__any_sync(0xffffffffu, bad)) break;
+            if (__any_sync(0xffffffffu, *(volatile int*)&B.sh->bail)) break;
+            if (spins >= B.sh->limit) {
                 *(volatile int*)&B.sh->bail = 1;
                 atomicExch(B.err, 1);
             }
@@ -617,7 +619,8 @@ __device__ __forceinline__ void res_step(const typename P::Args& a, const ResGeo
 // 64 registers a thread in 32-bit arithmetic, 168 in 64-bit: no phase spills
 template <class P>
 __global__ void __launch_bounds__(kResThreads(sizeof(typename P::R)), 1)
-    k_resident(typename P::Args a, ResGeom g, void* inboxes, const unsigned* __restrict__ base, int* err, int steps) {
+    k_resident(typename P::Args a, ResGeom g, void* inboxes, const unsigned* __restrict__ base, int* err, int limit,
+               int steps) {
     using L = typename P::L;
     using R = typename P::R;
     using T = typename P::T;
@@ -638,6 +641,7 @@ __global__ void __launch_bounds__(kResThreads(sizeof(typename P::R)), 1)
     const ResBox& b = B.b;
     if (threadIdx.x == 0) {
         sh.bail = 0;
+        sh.limit = limit;
         for (int c = 0; c < 3; ++c) sh.over[c] = 0;
     }
     B.syq = b.sy * L::Q;
@@ -770,8 +774,7 @@ __global__ void __launch_bounds__(kResThreads(sizeof(typename P::R)), 1)
 
 // launch with the arguments of a phase (returns the launch's error)
 template <class P>
-cudaError_t launch_resident(const typename P::Args& a, const ResPlan& p, void* inboxes, const unsigned* base, int* err,
-                            int steps, cudaStream_t s) {
+cudaError_t launch_resident(const typename P::Args& a, const ResPlan& p, const ResWords& w, int steps, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(k_resident<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -784,7 +787,7 @@ cudaError_t launch_resident(const typename P::Args& a, const ResPlan& p, void* i
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_resident<P>, a, p.g, inboxes, base, err, steps);
+    return cudaLaunchKernelEx(&cfg, k_resident<P>, a, p.g, w.inboxes, w.base, w.err, w.limit, steps);
 }
 
 }  // namespace lbm

@@ -234,34 +234,34 @@ long long resident_mismatches(int stencil, int nx, int ny, int nz) {
     return exchange_checks<float>(stencil, nx, ny, nz) + exchange_checks<double>(stencil, nx, ny, nz);
 }
 
-cudaError_t resident_flow_f64(int stencil, ResPhase ph, const FlowLaunch& a, const ResPlan& p, void* inboxes,
-                              const unsigned* base, int* err, int steps, cudaStream_t s);
-cudaError_t resident_thermal_f64(ResPhase ph, const ThermLaunch& a, const ResPlan& p, void* inboxes,
-                                 const unsigned* base, int* err, int steps, cudaStream_t s);
+cudaError_t resident_flow_f64(int stencil, ResPhase ph, const FlowLaunch& a, const ResPlan& p, const ResWords& w,
+                              int steps, cudaStream_t s);
+cudaError_t resident_thermal_f64(ResPhase ph, const ThermLaunch& a, const ResPlan& p, const ResWords& w,
+                                 int steps, cudaStream_t s);
 
-cudaError_t resident_flow(int stencil, int storage, ResPhase ph, const FlowLaunch& a, const ResPlan& p, void* inboxes,
-                          const unsigned* base, int* err, int steps, cudaStream_t s) {
+cudaError_t resident_flow(int stencil, int storage, ResPhase ph, const FlowLaunch& a, const ResPlan& p, const ResWords& w,
+                          int steps, cudaStream_t s) {
     using dispatch::flow_args;
-    if (storage == 0) return resident_flow_f64(stencil, ph, a, p, inboxes, base, err, steps, s);
+    if (storage == 0) return resident_flow_f64(stencil, ph, a, p, w, steps, s);
     if (ph == RP_FLOW) {
-        if (stencil == 0) return launch_resident<ResFlow<D2Q9, float, float, float>>(flow_args<1>(a), p, inboxes, base, err, steps, s);
-        if (storage == 1) return launch_resident<ResFlow<D3Q19, float, float, float>>(flow_args<1>(a), p, inboxes, base, err, steps, s);
-        if (storage == 2) return launch_resident<ResFlow<D3Q19, __half, float, float>>(flow_args<2>(a), p, inboxes, base, err, steps, s);
-        return launch_resident<ResFlow<D3Q19, __nv_bfloat16, float, float>>(flow_args<3>(a), p, inboxes, base, err, steps, s);
+        if (stencil == 0) return launch_resident<ResFlow<D2Q9, float, float, float>>(flow_args<1>(a), p, w, steps, s);
+        if (storage == 1) return launch_resident<ResFlow<D3Q19, float, float, float>>(flow_args<1>(a), p, w, steps, s);
+        if (storage == 2) return launch_resident<ResFlow<D3Q19, __half, float, float>>(flow_args<2>(a), p, w, steps, s);
+        return launch_resident<ResFlow<D3Q19, __nv_bfloat16, float, float>>(flow_args<3>(a), p, w, steps, s);
     }
     // the adjoint populations are FP32 in every 32-bit mode
     const auto x = flow_args<1>(a);
-    if (stencil == 0) return launch_resident<ResAdjoint<D2Q9, float, float, false>>(x, p, inboxes, base, err, steps, s);
-    if (ph == RP_ADJ) return launch_resident<ResAdjoint<D3Q19, float, float, false>>(x, p, inboxes, base, err, steps, s);
-    return launch_resident<ResAdjoint<D3Q19, float, float, true>>(x, p, inboxes, base, err, steps, s);
+    if (stencil == 0) return launch_resident<ResAdjoint<D2Q9, float, float, false>>(x, p, w, steps, s);
+    if (ph == RP_ADJ) return launch_resident<ResAdjoint<D3Q19, float, float, false>>(x, p, w, steps, s);
+    return launch_resident<ResAdjoint<D3Q19, float, float, true>>(x, p, w, steps, s);
 }
 
-cudaError_t resident_thermal(int storage, ResPhase ph, const ThermLaunch& a, const ResPlan& p, void* inboxes,
-                             const unsigned* base, int* err, int steps, cudaStream_t s) {
-    if (storage == 0) return resident_thermal_f64(ph, a, p, inboxes, base, err, steps, s);
+cudaError_t resident_thermal(int storage, ResPhase ph, const ThermLaunch& a, const ResPlan& p, const ResWords& w,
+                             int steps, cudaStream_t s) {
+    if (storage == 0) return resident_thermal_f64(ph, a, p, w, steps, s);
     const auto x = dispatch::therm_args<1>(a);
-    if (ph == RP_THERM) return launch_resident<ResHeat<float, float, float>>(x, p, inboxes, base, err, steps, s);
-    return launch_resident<ResHeatAdjoint<float, float>>(x, p, inboxes, base, err, steps, s);
+    if (ph == RP_THERM) return launch_resident<ResHeat<float, float, float>>(x, p, w, steps, s);
+    return launch_resident<ResHeatAdjoint<float, float>>(x, p, w, steps, s);
 }
 
 }  // namespace lbm

@@ -92,6 +92,7 @@ struct lbm_ctx {
     unsigned* sync = nullptr;  // their step counter and error flag
     size_t inbox_bytes = 0;
     unsigned long long tags = 0;  // step numbers used since the counter was cleared
+    int wait_limit = kWaitLimit;  // polls after which a resident launch gives up waiting
     bool resident = false;
     long long launches = 0;  // kernels launched (lbm_launches)
 
@@ -288,7 +289,7 @@ bool resident_fits(const lbm_ctx* c, int ph, int steps) {
 // enqueue n plain steps of a phase as one resident launch
 cudaError_t enqueue_resident(lbm_ctx* c, int ph, int n, cudaStream_t s) {
     cudaError_t e = cudaSuccess;
-    int* err = (int*)(c->sync + 1);
+    const ResWords w = {c->inbox, c->sync, (int*)(c->sync + 1), c->wait_limit};
     const ResPlan& p = c->plan[ph];
     if (ph == PH_FLOW || ph == PH_ADJ) {
         FlowLaunch a = flow_base(c);
@@ -297,7 +298,7 @@ cudaError_t enqueue_resident(lbm_ctx* c, int ph, int n, cudaStream_t s) {
         a.ain = c->fa[c->facur];
         a.aout = c->fa[1 - c->facur];
         const ResPhase rp = ph == PH_FLOW ? RP_FLOW : (c->thermal ? RP_ADJ_T : RP_ADJ);
-        e = resident_flow(c->stencil, c->storage, rp, a, p, c->inbox, c->sync, err, n, s);
+        e = resident_flow(c->stencil, c->storage, rp, a, p, w, n, s);
         (ph == PH_FLOW ? c->fcur : c->facur) ^= 1;
     } else {
         ThermLaunch a = therm_base(c);
@@ -305,7 +306,7 @@ cudaError_t enqueue_resident(lbm_ctx* c, int ph, int n, cudaStream_t s) {
         a.gout = c->g[1 - c->gcur];
         a.ain = c->ga[c->gacur];
         a.aout = c->ga[1 - c->gacur];
-        e = resident_thermal(c->storage, ph == PH_THERM ? RP_THERM : RP_TADJ, a, p, c->inbox, c->sync, err, n, s);
+        e = resident_thermal(c->storage, ph == PH_THERM ? RP_THERM : RP_TADJ, a, p, w, n, s);
         (ph == PH_THERM ? c->gcur : c->gacur) ^= 1;
     }
     return e;
@@ -1230,6 +1231,22 @@ size_t state_size(lbm_ctx* c) {
 extern "C" {
 
 long long lbm_launches(lbm_ctx* c) { return c ? c->launches : 0; }
+
+lbm_status lbm_set_resident(lbm_ctx* c, int wait_limit, unsigned step_number) {
+    if (!c) return fail(LBM_ERR_ARG, "ctx is null");
+    if (wait_limit < 0) return fail(LBM_ERR_ARG, "wait_limit < 0");
+    if (!c->inbox) return LBM_OK;
+    lbm_status st = enter(c);
+    if (st != LBM_OK) return st;
+    const unsigned sync[2] = {step_number, 0};
+    CUDA_TRY(cudaMemsetAsync(c->inbox, 0, c->inbox_bytes, c->stream));
+    CUDA_TRY(cudaMemcpyAsync(c->sync, sync, sizeof(sync), cudaMemcpyHostToDevice, c->stream));
+    CUDA_TRY(cudaStreamSynchronize(c->stream));
+    c->tags = step_number;
+    if (c->wait_limit != wait_limit) c->drop_graphs();  // the launches hold it
+    c->wait_limit = wait_limit;
+    return leave(c);
+}
 
 size_t lbm_state_bytes(lbm_ctx* c) { return c ? state_size(c) : 0; }
 

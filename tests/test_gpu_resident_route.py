@@ -1,0 +1,86 @@
+"""Which route the steps of a solve take, and what happens when a resident
+launch cannot be finished.
+
+Results are the same bit for bit on every route, so the route itself is read
+from the launch counter: a block of k steps with its finalize kernel is k + 1
+launches, or 3 when its plain steps are one resident launch.
+"""
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2501_02161_gb300 import _capi as C
+from paper_2501_02161_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+WAIT = 1 << 21  # polls of a wait, as the library has it by default
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2501_02161_gb300 import build as B
+    B.build()
+
+
+def solver(lat, storage="fp32"):
+    from paper_2501_02161_gb300.solver import Solver
+    return Solver.from_lattice(lat, storage=storage)
+
+
+def set_resident(s, wait_limit=WAIT, step_number=0):
+    C.check(s.lib.lbm_set_resident(s._ctx, wait_limit, step_number), "lbm_set_resident")
+
+
+def solve(s, steps, check):
+    rf = s.forward(tol=0, max_steps=steps, check_every=check)
+    ra = s.adjoint(tol=0, max_steps=steps, check_every=check)
+    fs, gs = s.adjoint_fields()
+    out = [torch.tensor([rf.J, rf.I, ra.I], dtype=torch.float64), *s.fields(), fs, gs, s.sensitivity()]
+    return [x.cpu() for x in out if x is not None]
+
+
+def same(got, ref):
+    for a, b in zip(got, ref):
+        assert torch.isfinite(b).all()
+        assert torch.equal(a, b)
+
+
+LATTICES = {
+    "bend_24": lambda: I.pipe_bend_3d(24, width=6, re=15.0, seed=1),
+    "bend2d_64": lambda: I.pipe_bend_2d(64, 64, width=16),
+    "quarter_45x24x13": lambda: I.heat_sink_quarter(45, 24, 13),
+}
+
+
+@pytest.mark.parametrize("storage", ["fp32", "fp64"])
+@pytest.mark.parametrize("name", LATTICES)
+def test_a_wait_that_gives_up_is_made_good(name, storage):
+    """With a limit of 0 polls a wait gives up at the first word that is not
+    there yet; the kernel ends by itself, its block runs again a launch per
+    step from the untouched input, and nothing of it is left in the results."""
+    s = solver(LATTICES[name](), storage)
+    ref = solve(s, 200, 5)
+    set_resident(s, wait_limit=0)
+    n = s.launches()
+    same(solve(s, 200, 100), ref)
+    phases = 4 if s.thermal else 2
+    # every phase's two blocks a launch per step, and the launches that gave up beside them
+    assert s.launches() - n > phases * 2 * 101 + 3
+    s.close()
+
+
+@pytest.mark.parametrize("start", [0xF0000000 - 70, 0xFFFFFFF0])
+def test_step_numbers_start_again(start):
+    """The words carry 32-bit step numbers: before they run out the inboxes are
+    cleared and the count begins again."""
+    s = solver(LATTICES["bend_24"]())
+    ref = solve(s, 400, 5)
+    set_resident(s, step_number=start)
+    n = s.launches()
+    same(solve(s, 400, 100), ref)
+    # initial populations and four blocks per phase, and dJ/dgamma
+    assert s.launches() - n == 2 * (1 + 4 * 3) + 1
+    s.close()
