@@ -5,6 +5,9 @@ Results are the same bit for bit on every route, so the route itself is read
 from the launch counter: a block of k steps with its finalize kernel is k + 1
 launches, or 3 when its plain steps are one resident launch.
 """
+import threading
+import time
+
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -84,3 +87,34 @@ def test_step_numbers_start_again(start):
     # initial populations and four blocks per phase, and dJ/dgamma
     assert s.launches() - n == 2 * (1 + 4 * 3) + 1
     s.close()
+
+
+def test_solves_beside_one_another_step_by_launches():
+    """A resident launch would keep the other context's steps waiting for a
+    whole block: while a second context is in a solve both go a launch per step."""
+    s, other = solver(LATTICES["bend_24"]()), solver(I.pipe_bend_3d(64, width=16, re=20.0, seed=2))
+    ref = solve(s, 400, 100)
+    n = s.launches()
+    same(solve(s, 400, 100), ref)
+    assert s.launches() - n == 2 * (1 + 4 * 3) + 1  # alone: resident
+    torch.cuda.synchronize()
+
+    def long_solve():
+        with torch.cuda.stream(torch.cuda.Stream()):
+            other.forward(tol=0, max_steps=200000, check_every=500)
+
+    t = threading.Thread(target=long_solve)
+    began = other.launches()
+    t.start()
+    while other.launches() < began + 10:
+        time.sleep(0.001)
+    n = s.launches()
+    with torch.cuda.stream(torch.cuda.Stream()):
+        got = solve(s, 400, 100)
+    n = s.launches() - n
+    beside = t.is_alive()
+    t.join()
+    assert beside and n == 2 * (1 + 4 * 101) + 1
+    same(got, ref)
+    s.close()
+    other.close()
