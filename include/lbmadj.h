@@ -312,7 +312,8 @@ long long lbm_launches(lbm_ctx* ctx);
 /* How the context's resident launches wait and count (no effect on a lattice
  * that has none): wait_limit, the polls after which a wait gives up and the
  * steps run again a launch each (by default 2^21, about a second; 0: a word
- * that is not there at the first poll is given up), and step_number, from which
+ * that is not there at the first poll is given up; the third time the context
+ * stays with a launch per step, until this call), and step_number, from which
  * the steps are numbered on (they start again from 0 before 2^32).  For tests
  * of what a waiting block and a long run do: ordinary programs have no use for
  * it.  Errors: LBM_ERR_ARG (null, wait_limit < 0). */

@@ -94,6 +94,7 @@ struct lbm_ctx {
     unsigned long long tags = 0;  // step numbers used since the counter was cleared
     int wait_limit = kWaitLimit;  // polls after which a resident launch gives up waiting
     bool resident = false;
+    int gave_up = 0;         // resident launches that were refused or gave up waiting
     long long launches = 0;  // kernels launched (lbm_launches)
 
     Geom geom{};
@@ -281,8 +282,14 @@ int& parity_of(lbm_ctx* c, int ph) {
 // set-up and the global passes at its ends cost about three steps).
 constexpr int kResidentMinSteps = 6;
 
+// A launch that gave up has cost its context a wait of about a second.  What
+// held it up may be over by the next block (another process's work on the
+// device) or may be there for good: the third time the context stays with a
+// launch per step.
+constexpr int kResidentTries = 3;
+
 bool resident_fits(const lbm_ctx* c, int ph, int steps) {
-    return c->resident && c->plan[ph].ok && steps >= kResidentMinSteps &&
+    return c->resident && c->gave_up < kResidentTries && c->plan[ph].ok && steps >= kResidentMinSteps &&
            !(ph == PH_ADJ && c->adj_scheme == LBM_ADJOINT_CONTINUOUS);
 }
 
@@ -404,7 +411,8 @@ lbm_status run_block_sync(lbm_ctx* c, int ph, int k, const InFlight& solve) {
         // the launch was refused, or a wait gave up (the block's input is
         // untouched and its reducing step was left out): the block runs
         // again, a launch per step
-        c->resident = false;
+        ++c->gave_up;
+        CUDA_TRY(cudaMemsetAsync(c->sync + 1, 0, sizeof(unsigned), c->stream));
     }
     lbm_status st = run_block(c, ph, k, false);
     if (st != LBM_OK) return st;
@@ -1256,6 +1264,7 @@ lbm_status lbm_set_resident(lbm_ctx* c, int wait_limit, unsigned step_number) {
     CUDA_TRY(cudaMemcpyAsync(c->sync, sync, sizeof(sync), cudaMemcpyHostToDevice, c->stream));
     CUDA_TRY(cudaStreamSynchronize(c->stream));
     c->tags = step_number;
+    c->gave_up = 0;
     if (c->wait_limit != wait_limit) c->drop_graphs();  // the launches hold it
     c->wait_limit = wait_limit;
     return leave(c);
@@ -1397,7 +1406,8 @@ lbm_status lbm_time_steps(lbm_ctx* c, int phase, int n, double* ms_per_step) {
         CUDA_TRY(cudaMemcpyAsync(c->hres, c->dres, sizeof(double) * 3, cudaMemcpyDeviceToHost, c->stream));
         CUDA_TRY(cudaStreamSynchronize(c->stream));
         if (c->hres[2] != 0.0) {
-            c->resident = false;
+            ++c->gave_up;
+            CUDA_TRY(cudaMemsetAsync(c->sync + 1, 0, sizeof(unsigned), c->stream));
             (phase == PH_FLOW || phase == PH_THERM ? c->fstate : c->astate) = false;
             return fail(LBM_ERR_CUDA, "a resident launch gave up waiting");
         }

@@ -118,3 +118,23 @@ def test_solves_beside_one_another_step_by_launches():
     same(got, ref)
     s.close()
     other.close()
+
+
+def test_a_context_tries_again_after_a_wait_gave_up():
+    """One stall does not turn a context slow for good; the third time it stays
+    with a launch per step."""
+    s = solver(LATTICES["bend_24"]())
+    init, block, resident = 1, 101, 3
+
+    def forward(blocks):
+        n = s.launches()
+        s.forward(tol=0, max_steps=100 * blocks, check_every=100)
+        return s.launches() - n
+
+    set_resident(s, wait_limit=0)
+    assert forward(2) == init + 2 * (resident + block)
+    assert forward(3) == init + (resident + block) + 2 * block
+    assert forward(3) == init + 3 * block
+    set_resident(s)
+    assert forward(3) == init + 3 * resident
+    s.close()
