@@ -355,12 +355,12 @@ struct InFlight {
 };
 
 // step numbers are 32 bits: start again from cleared inboxes before they run out
-lbm_status resident_tags(lbm_ctx* c, int k) {
-    c->tags += (unsigned)k;
+lbm_status resident_tags(lbm_ctx* c, long long k) {
+    c->tags += k;
     if (c->tags > 0xF0000000ull) {
         CUDA_TRY(cudaMemsetAsync(c->inbox, 0, c->inbox_bytes, c->stream));
         CUDA_TRY(cudaMemsetAsync(c->sync, 0, 2 * sizeof(unsigned), c->stream));
-        c->tags = (unsigned)k;
+        c->tags = k;
     }
     return LBM_OK;
 }
@@ -393,7 +393,7 @@ lbm_status run_block(lbm_ctx* c, int ph, int k, bool resident) {
         if (st != LBM_OK) return st;
     }
     CUDA_TRY(cudaGraphLaunch(it->second, c->stream));
-    c->launches += resident ? 3 : k + 1;  // steps, reducing step, finalize
+    c->launches += resident ? 3 : 1 + (long long)k;  // steps, reducing step, finalize
     // a launch swaps the buffers: once per step, once per resident launch
     if (!resident && k % 2) par ^= 1;
     return LBM_OK;
@@ -417,6 +417,58 @@ lbm_status run_block_sync(lbm_ctx* c, int ph, int k, const InFlight& solve) {
     lbm_status st = run_block(c, ph, k, false);
     if (st != LBM_OK) return st;
     CUDA_TRY(cudaStreamSynchronize(c->stream));
+    return LBM_OK;
+}
+
+// the graph and events of one timing, given back on every way out
+struct Timing {
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    ~Timing() {
+        if (graph) cudaGraphDestroy(graph);
+        if (exec) cudaGraphExecDestroy(exec);
+        if (e0) cudaEventDestroy(e0);
+        if (e1) cudaEventDestroy(e1);
+    }
+};
+
+// capture m plain steps of a phase (resident: as two launches, an even count of
+// them, too), replay them once untimed (began is set) and once timed
+lbm_status time_replay(lbm_ctx* c, int ph, long long m, bool resident, bool* began, float* ms) {
+    Timing t;
+    int& par = parity_of(c, ph);
+    const int par0 = par;
+    CUDA_TRY(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
+    cudaError_t e = cudaSuccess;
+    if (resident) {
+        for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
+            e = enqueue_resident(c, ph, (int)(m / 2), c->stream);
+            if (e == cudaSuccess) e = finalize_launch(c->partials, 0, 1, c->dres, c->stream, c->sync, (int)(m / 2));
+        }
+    } else {
+        for (long long i = 0; i < m && e == cudaSuccess; ++i) e = enqueue_step(c, ph, false, c->stream);
+    }
+    const cudaError_t e2 = cudaStreamEndCapture(c->stream, &t.graph);
+    par = par0;
+    if (e != cudaSuccess || e2 != cudaSuccess) {
+        (void)cudaGetLastError();
+        return fail(LBM_ERR_CUDA, "time_steps capture failed");
+    }
+    CUDA_TRY(cudaGraphInstantiate(&t.exec, t.graph, 0));
+    CUDA_TRY(cudaEventCreate(&t.e0));
+    CUDA_TRY(cudaEventCreate(&t.e1));
+    if (resident) {
+        const lbm_status st = resident_tags(c, 2 * m);
+        if (st != LBM_OK) return st;
+    }
+    CUDA_TRY(cudaGraphLaunch(t.exec, c->stream));  // untimed: first replay uploads the graph
+    *began = true;
+    CUDA_TRY(cudaEventRecord(t.e0, c->stream));
+    CUDA_TRY(cudaGraphLaunch(t.exec, c->stream));
+    CUDA_TRY(cudaEventRecord(t.e1, c->stream));
+    CUDA_TRY(cudaEventSynchronize(t.e1));
+    CUDA_TRY(cudaEventElapsedTime(ms, t.e0, t.e1));
     return LBM_OK;
 }
 
@@ -1361,47 +1413,24 @@ lbm_status lbm_time_steps(lbm_ctx* c, int phase, int n, double* ms_per_step) {
         return fail(LBM_ERR_ARG, "temperature phase without the thermal lattice");
     if (phase != PH_FLOW && !c->fwd_done) return fail(LBM_ERR_ORDER, "needs a completed lbm_forward");
     if ((st = enter(c)) != LBM_OK) return st;
-    const int m = n + (n & 1);  // an even count keeps the buffer parity
+    const long long m = (long long)n + (n & 1);  // an even count keeps the buffer parity
     const InFlight solve(c->device);
-    const bool resident = resident_fits(c, phase, m / 2) && solve.alone();
-    int& par = parity_of(c, phase);
-    const int par0 = par;
-    cudaGraph_t graph = nullptr;
-    CUDA_TRY(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = cudaSuccess;
-    if (resident) {
-        for (int i = 0; i < 2 && e == cudaSuccess; ++i) {  // an even count of launches, too
-            e = enqueue_resident(c, phase, m / 2, c->stream);
-            if (e == cudaSuccess) e = finalize_launch(c->partials, 0, 1, c->dres, c->stream, c->sync, m);
-        }
-    } else {
-        for (int i = 0; i < m && e == cudaSuccess; ++i) e = enqueue_step(c, phase, false, c->stream);
-    }
-    cudaError_t e2 = cudaStreamEndCapture(c->stream, &graph);
-    par = par0;
-    if (e != cudaSuccess || e2 != cudaSuccess) {
-        if (graph) cudaGraphDestroy(graph);
-        (void)cudaGetLastError();
-        return fail(LBM_ERR_CUDA, "time_steps capture failed");
-    }
-    cudaGraphExec_t exec = nullptr;
-    e = cudaGraphInstantiate(&exec, graph, 0);
-    cudaGraphDestroy(graph);
-    CUDA_TRY(e);
-    if (resident && (st = resident_tags(c, 4 * m)) != LBM_OK) return st;
-    cudaEvent_t e0, e1;
-    CUDA_TRY(cudaEventCreate(&e0));
-    CUDA_TRY(cudaEventCreate(&e1));
-    CUDA_TRY(cudaGraphLaunch(exec, c->stream));  // untimed: first replay uploads the graph
-    CUDA_TRY(cudaEventRecord(e0, c->stream));
-    CUDA_TRY(cudaGraphLaunch(exec, c->stream));
-    CUDA_TRY(cudaEventRecord(e1, c->stream));
-    CUDA_TRY(cudaEventSynchronize(e1));
     float ms = 0.f;
-    CUDA_TRY(cudaEventElapsedTime(&ms, e0, e1));
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    cudaGraphExecDestroy(exec);
+    bool began = false;
+    // (the step numbers of all replays stay below the restart's threshold)
+    const bool resident = m <= 1 << 28 && resident_fits(c, phase, (int)(m / 2)) && solve.alone();
+    if (resident) {
+        st = time_replay(c, phase, m, true, &began, &ms);
+        if (st != LBM_OK && !began) {  // refused: nothing has run
+            (void)cudaGetLastError();
+            ++c->gave_up;
+        }
+    }
+    if (!began) st = time_replay(c, phase, m, false, &began, &ms);
+    if (st != LBM_OK) {
+        (void)cudaStreamSynchronize(c->stream);
+        return st;
+    }
     if (resident) {
         CUDA_TRY(cudaMemcpyAsync(c->hres, c->dres, sizeof(double) * 3, cudaMemcpyDeviceToHost, c->stream));
         CUDA_TRY(cudaStreamSynchronize(c->stream));

@@ -138,3 +138,23 @@ def test_a_context_tries_again_after_a_wait_gave_up():
     set_resident(s)
     assert forward(3) == init + 3 * resident
     s.close()
+
+
+@pytest.mark.parametrize("storage", ["fp32", "fp64"])
+@pytest.mark.parametrize("n", [9, 400])
+def test_timed_steps_advance_a_phase_as_a_solve_does(n, storage):
+    """2 n steps (n rounded up to even) in either route."""
+    for name in ("bend_24", "quarter_45x24x13"):
+        s, ref = solver(LATTICES[name](), storage), solver(LATTICES[name](), storage)
+        for x in (s, ref):
+            x.forward(tol=0, max_steps=20, check_every=5)
+            x.adjoint(tol=0, max_steps=20, check_every=5)
+        steps = 2 * (n + n % 2)
+        assert s.time_steps(0, n) > 0
+        # the reducing step that ends a solve gives the fields
+        s.forward(tol=0, max_steps=1, check_every=1, reset=False)
+        ref.forward(tol=0, max_steps=steps, check_every=5, reset=False)
+        ref.forward(tol=0, max_steps=1, check_every=1, reset=False)
+        same(s.fields()[:2], ref.fields()[:2])
+        s.close()
+        ref.close()
