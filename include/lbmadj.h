@@ -300,7 +300,8 @@ lbm_status lbm_get_adjoint(lbm_ctx* ctx, void* fstar, void* gstar, int dtype, in
  * gaps between graph nodes).  phase: 0 flow forward, 1 temperature forward, 2 flow adjoint,
  * 3 temperature adjoint.  The 2n steps advance that phase's state as a solve
  * would; no reduction runs.  Needs the inputs set (LBM_ERR_ORDER) and, for
- * phases 1-3, a completed lbm_forward. */
+ * phases 1-3, a completed lbm_forward.  After LBM_ERR_CUDA from a wait that gave
+ * up, the phase and those after it have to be solved again. */
 lbm_status lbm_time_steps(lbm_ctx* ctx, int phase, int n, double* ms_per_step);
 
 /* Kernels that the context's initialisations, solves and sensitivities have

@@ -1437,7 +1437,13 @@ lbm_status lbm_time_steps(lbm_ctx* c, int phase, int n, double* ms_per_step) {
         if (c->hres[2] != 0.0) {
             ++c->gave_up;
             CUDA_TRY(cudaMemsetAsync(c->sync + 1, 0, sizeof(unsigned), c->stream));
-            (phase == PH_FLOW || phase == PH_THERM ? c->fstate : c->astate) = false;
+            // both buffers of the phase have been written: nothing that builds on
+            // its state stands
+            if (phase == PH_FLOW || phase == PH_THERM)
+                c->fstate = c->flow_done = c->fwd_done = false;
+            else
+                c->astate = false;
+            c->tadj_done = c->adj_done = false;
             return fail(LBM_ERR_CUDA, "a resident launch gave up waiting");
         }
     }

@@ -158,3 +158,27 @@ def test_timed_steps_advance_a_phase_as_a_solve_does(n, storage):
         same(s.fields()[:2], ref.fields()[:2])
         s.close()
         ref.close()
+
+
+@pytest.mark.parametrize("phase", [0, 1, 2, 3])
+def test_timed_steps_that_gave_up_leave_nothing_to_read(phase):
+    """Both buffers of the phase have been written: what builds on it is refused
+    until it has been solved again, and then right."""
+    s = solver(LATTICES["quarter_45x24x13"]())
+    ref = solve(s, 40, 5)
+    set_resident(s, wait_limit=0)
+    with pytest.raises(C.LBMError):
+        s.time_steps(phase, 400)
+    set_resident(s)
+    with pytest.raises(C.LBMError):
+        s.sensitivity()
+    with pytest.raises(C.LBMError):
+        s.adjoint_fields()
+    if phase < 2:
+        with pytest.raises(C.LBMError):
+            s.fields()
+        s.forward(tol=0, max_steps=40, check_every=5, reset=False)
+    s.adjoint(tol=0, max_steps=40, check_every=5, reset=phase < 2)
+    fs, gs = s.adjoint_fields()
+    same([x.cpu() for x in (*s.fields(), fs, gs, s.sensitivity())], ref[1:])
+    s.close()
