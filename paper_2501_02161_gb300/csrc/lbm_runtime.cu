@@ -433,8 +433,9 @@ struct Timing {
     }
 };
 
-// capture m plain steps of a phase (resident: as two launches, an even count of
-// them, too), replay them once untimed (began is set) and once timed
+// capture m plain steps of a phase, replay them once untimed (began is set) and
+// once timed.  Resident: two launches, each with a one-step launch after it as in
+// a solve (the temperature adjoint's leaves its outflow values for the coupling)
 lbm_status time_replay(lbm_ctx* c, int ph, long long m, bool resident, bool* began, float* ms) {
     Timing t;
     int& par = parity_of(c, ph);
@@ -443,7 +444,8 @@ lbm_status time_replay(lbm_ctx* c, int ph, long long m, bool resident, bool* beg
     cudaError_t e = cudaSuccess;
     if (resident) {
         for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
-            e = enqueue_resident(c, ph, (int)(m / 2), c->stream);
+            e = enqueue_resident(c, ph, (int)(m / 2) - 1, c->stream);
+            if (e == cudaSuccess) e = enqueue_step(c, ph, false, c->stream);
             if (e == cudaSuccess) e = finalize_launch(c->partials, 0, 1, c->dres, c->stream, c->sync, (int)(m / 2));
         }
     } else {
@@ -1418,7 +1420,7 @@ lbm_status lbm_time_steps(lbm_ctx* c, int phase, int n, double* ms_per_step) {
     float ms = 0.f;
     bool began = false;
     // (the step numbers of all replays stay below the restart's threshold)
-    const bool resident = m <= 1 << 28 && resident_fits(c, phase, (int)(m / 2)) && solve.alone();
+    const bool resident = m <= 1 << 28 && resident_fits(c, phase, (int)(m / 2) - 1) && solve.alone();
     if (resident) {
         st = time_replay(c, phase, m, true, &began, &ms);
         if (st != LBM_OK && !began) {  // refused: nothing has run

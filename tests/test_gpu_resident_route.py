@@ -182,3 +182,20 @@ def test_timed_steps_that_gave_up_leave_nothing_to_read(phase):
     fs, gs = s.adjoint_fields()
     same([x.cpu() for x in (*s.fields(), fs, gs, s.sensitivity())], ref[1:])
     s.close()
+
+
+def test_timed_temperature_adjoint_leaves_the_coupling_its_values():
+    """The coupling of the flow adjoint reads what a step of the temperature
+    adjoint leaves at outflow nodes beside the populations."""
+    s, ref = (solver(LATTICES["quarter_45x24x13"]()) for _ in range(2))
+    for x in (s, ref):
+        x.forward(tol=0, max_steps=40, check_every=5)
+        x.adjoint(tol=0, max_steps=40, check_every=5)
+    s.time_steps(3, 400)
+    s.solve_phase(3, tol=0, max_steps=0, check_every=5, reset=False)  # the coupling alone
+    ref.solve_phase(3, tol=0, max_steps=800, check_every=5, reset=False)
+    for x in (s, ref):
+        x.solve_phase(2, tol=0, max_steps=20, check_every=5, reset=False)
+    same([*s.adjoint_fields(), s.sensitivity()], [*ref.adjoint_fields(), ref.sensitivity()])
+    s.close()
+    ref.close()
