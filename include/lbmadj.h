@@ -310,15 +310,17 @@ lbm_status lbm_time_steps(lbm_ctx* ctx, int phase, int n, double* ms_per_step);
  * inputs and outputs, lbm_time_steps and packed batch launches are not counted. */
 long long lbm_launches(lbm_ctx* ctx);
 
-/* How the context's resident launches wait and count (no effect on a lattice
- * that has none): wait_limit, the polls after which a wait gives up and the
- * steps run again a launch each (by default 2^21, about a second; 0: a word
- * that is not there at the first poll is given up; the third time the context
- * stays with a launch per step, until this call), and step_number, from which
- * the steps are numbered on (they start again from 0 before 2^32).  For tests
- * of what a waiting block and a long run do: ordinary programs have no use for
- * it.  Errors: LBM_ERR_ARG (null, wait_limit < 0). */
-lbm_status lbm_set_resident(lbm_ctx* ctx, int wait_limit, unsigned step_number);
+/* When the context's plain steps go resident, and how such launches wait and
+ * count (no effect on a lattice that has none): min_steps, the plain steps of a
+ * block from which on they are one resident launch (by default 0: where that
+ * was measured to take no longer than a launch per step); wait_limit, the polls
+ * after which a wait gives up and the steps run again a launch each (by default
+ * 2^21, about a second; 0: a word that is not there at the first poll is given
+ * up; the third time the context stays with a launch per step, until this
+ * call); step_number, from which the steps are numbered on (they start again
+ * from 0 before 2^32).  For tests of what a short launch, a waiting block and a
+ * long run do: ordinary programs have no use for it.  Errors: LBM_ERR_ARG (null, a negative argument). */
+lbm_status lbm_set_resident(lbm_ctx* ctx, int min_steps, int wait_limit, unsigned step_number);
 
 /* ---------------------------------------------------------------------------
  * Checkpoint / resume of a context's solver state (no counterpart in the

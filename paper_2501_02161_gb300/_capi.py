@@ -93,7 +93,7 @@ SIGNATURES = {
     "lbm_get_adjoint": (_I, [_VP, _VP, _VP, _I, _I]),
     "lbm_time_steps": (_I, [_VP, _I, _I, ctypes.POINTER(ctypes.c_double)]),
     "lbm_launches": (ctypes.c_longlong, [_VP]),
-    "lbm_set_resident": (_I, [_VP, _I, ctypes.c_uint]),
+    "lbm_set_resident": (_I, [_VP, _I, _I, ctypes.c_uint]),
     "lbm_flow_step_noalloc": (_I, [ctypes.POINTER(lbm_step_desc), _VP]),
     "lbm_footprint_bytes": (ctypes.c_size_t, [_I, _I, _I, _I, _I, _I]),
     "lbm_batch_create": (_I, [ctypes.POINTER(_VP), _I, _I, _I, _SZ]),

@@ -92,6 +92,7 @@ struct lbm_ctx {
     unsigned* sync = nullptr;  // their step counter and error flag
     size_t inbox_bytes = 0;
     unsigned long long tags = 0;  // step numbers used since the counter was cleared
+    int min_steps = 0;       // plain steps that go resident (0: resident_min_steps)
     int wait_limit = kWaitLimit;  // polls after which a resident launch gives up waiting
     bool resident = false;
     int gave_up = 0;         // resident launches that were refused or gave up waiting
@@ -278,9 +279,25 @@ int& parity_of(lbm_ctx* c, int ph) {
     return ph == PH_FLOW ? c->fcur : (ph == PH_THERM ? c->gcur : (ph == PH_ADJ ? c->facur : c->gacur));
 }
 
-// A resident launch beats a launch per step from a handful of steps on (its
-// set-up and the global passes at its ends cost about three steps).
-constexpr int kResidentMinSteps = 6;
+// Plain steps from which on one resident launch takes no longer than a launch
+// for each.  The set-up of a resident launch (20 us at 16^3, 27 at 32^3, 50 at
+// 48^3, 92 at 64^3: it lists the nodes of a box) has to be made good by what a
+// step saves, measured over 21 lattices with blocks of 6 to 400 steps:
+//  - 64-bit arithmetic saves 4 to 38 us a step: 0.57-0.87 of the time from 6 steps on;
+//  - the temperature phases break even at 16 to 40 steps;
+//  - the flow phases at 17 to 38 (forward and adjoint of 12^3: 50 and 26), and at
+//    55 to 70 (32^3, 64^3; thermal 128 x 64 x 32: 58 and 40) where rows are multiples
+//    of 32 nodes, at which a launch per step is at its best;
+//  - the 16-bit forward step over pairs of nodes is the fastest launch per step:
+//    32^3 28 steps, 64^3 120, so it grows with the nodes of a box.
+int resident_min_steps(const lbm_ctx* c, int ph) {
+    if (c->min_steps > 0) return c->min_steps;
+    if (c->storage == LBM_FP64) return 6;
+    if (ph == PH_THERM || ph == PH_TADJ) return 36;
+    if (ph == PH_FLOW && c->storage != LBM_FP32 && c->nx % 2 == 0 && !c->mirror)
+        return 16 + c->plan[ph].g.bx * c->plan[ph].g.by * c->plan[ph].g.bz / 16;
+    return c->nx % 32 == 0 ? 56 : 36;
+}
 
 // A launch that gave up has cost its context a wait of about a second.  What
 // held it up may be over by the next block (another process's work on the
@@ -289,7 +306,8 @@ constexpr int kResidentMinSteps = 6;
 constexpr int kResidentTries = 3;
 
 bool resident_fits(const lbm_ctx* c, int ph, int steps) {
-    return c->resident && c->gave_up < kResidentTries && c->plan[ph].ok && steps >= kResidentMinSteps &&
+    return c->resident && c->gave_up < kResidentTries && c->plan[ph].ok &&
+           steps >= resident_min_steps(c, ph) &&
            !(ph == PH_ADJ && c->adj_scheme == LBM_ADJOINT_CONTINUOUS);
 }
 
@@ -1307,9 +1325,10 @@ extern "C" {
 
 long long lbm_launches(lbm_ctx* c) { return c ? c->launches : 0; }
 
-lbm_status lbm_set_resident(lbm_ctx* c, int wait_limit, unsigned step_number) {
+lbm_status lbm_set_resident(lbm_ctx* c, int min_steps, int wait_limit, unsigned step_number) {
     if (!c) return fail(LBM_ERR_ARG, "ctx is null");
-    if (wait_limit < 0) return fail(LBM_ERR_ARG, "wait_limit < 0");
+    if (min_steps < 0 || wait_limit < 0) return fail(LBM_ERR_ARG, "negative argument");
+    c->min_steps = min_steps;
     if (!c->inbox) return LBM_OK;
     lbm_status st = enter(c);
     if (st != LBM_OK) return st;

@@ -33,8 +33,8 @@ def solver(lat, storage="fp32"):
     return Solver.from_lattice(lat, storage=storage)
 
 
-def set_resident(s, wait_limit=WAIT, step_number=0):
-    C.check(s.lib.lbm_set_resident(s._ctx, wait_limit, step_number), "lbm_set_resident")
+def set_resident(s, min_steps=0, wait_limit=WAIT, step_number=0):
+    C.check(s.lib.lbm_set_resident(s._ctx, min_steps, wait_limit, step_number), "lbm_set_resident")
 
 
 def solve(s, steps, check):
@@ -53,13 +53,15 @@ def same(got, ref):
 
 LATTICES = {
     "bend_24": lambda: I.pipe_bend_3d(24, width=6, re=15.0, seed=1),
+    "bend_32": lambda: I.pipe_bend_3d(32, width=8, re=15.0, seed=1),
+    "bend_33": lambda: I.pipe_bend_3d(33, width=8, re=15.0, seed=1),
     "bend2d_64": lambda: I.pipe_bend_2d(64, 64, width=16),
     "quarter_45x24x13": lambda: I.heat_sink_quarter(45, 24, 13),
 }
 
 
 @pytest.mark.parametrize("storage", ["fp32", "fp64"])
-@pytest.mark.parametrize("name", LATTICES)
+@pytest.mark.parametrize("name", ["bend_24", "bend2d_64", "quarter_45x24x13"])
 def test_a_wait_that_gives_up_is_made_good(name, storage):
     """With a limit of 0 polls a wait gives up at the first word that is not
     there yet; the kernel ends by itself, its block runs again a launch per
@@ -199,3 +201,58 @@ def test_timed_temperature_adjoint_leaves_the_coupling_its_values():
     same([*s.adjoint_fields(), s.sensitivity()], [*ref.adjoint_fields(), ref.sensitivity()])
     s.close()
     ref.close()
+
+
+@pytest.mark.parametrize("name,storage,first", [
+    ("bend_24", "fp32", {0: 36, 2: 36}),
+    ("bend_32", "fp32", {0: 56, 2: 56}),
+    ("bend_24", "fp64", {0: 6, 2: 6}),
+    ("bend_32", "fp64", {0: 6, 2: 6}),
+    ("bend2d_64", "fp32", {0: 56, 2: 56}),
+    ("quarter_45x24x13", "fp32", {0: 36, 1: 36, 2: 36, 3: 36}),
+    ("bend_33", "bf16", {0: 36, 2: 36}),
+])
+def test_short_blocks_keep_a_launch_per_step(name, storage, first):
+    """The set-up of a resident launch takes 20 to 100 us: blocks with too few
+    plain steps to make it good step by launches."""
+    s = solver(LATTICES[name](), storage)
+    s.forward(tol=0, max_steps=4, check_every=2)
+    s.adjoint(tol=0, max_steps=4, check_every=2)
+    for phase, steps in sorted(first.items(), key=lambda v: (0, 1, 3, 2).index(v[0])):
+        for plain, launches in ((steps - 1, steps + 1), (steps, 3)):
+            n = s.launches()
+            s.solve_phase(phase, tol=0, max_steps=2 * (plain + 1), check_every=plain + 1, reset=False)
+            # the temperature adjoint ends with the coupling
+            assert s.launches() - n - (phase == 3) == 2 * launches
+    s.close()
+
+
+def test_short_16_bit_blocks_keep_the_paired_step():
+    """The 16-bit forward step over pairs of nodes: the line lies with the box."""
+    s = solver(LATTICES["bend_32"](), "fp16")
+    s.forward(tol=0, max_steps=4, check_every=2)
+
+    def per_block(plain):
+        n = s.launches()
+        s.solve_phase(0, tol=0, max_steps=plain + 1, check_every=plain + 1, reset=False)
+        return s.launches() - n
+
+    assert per_block(19) == 21
+    assert per_block(60) == 3
+    s.close()
+
+
+@pytest.mark.parametrize("check", [2, 3, 4, 8, 15])
+@pytest.mark.parametrize("storage", ["fp32", "fp64", "bf16"])
+@pytest.mark.parametrize("name", ["bend_24", "quarter_45x24x13"])
+def test_resident_launches_of_few_steps(name, storage, check):
+    """One to fourteen steps in a launch, both parities."""
+    s = solver(LATTICES[name](), storage)
+    ref = solve(s, 60, 1)
+    set_resident(s, min_steps=1)
+    n = s.launches()
+    same(solve(s, 60, check), ref)
+    phases = 4 if s.thermal else 2
+    # initial populations (the temperature's also collide), blocks, coupling, dJ/dgamma
+    assert s.launches() - n == phases + 2 * (phases == 4) + phases * -(-60 // check) * 3 + 1
+    s.close()
