@@ -18,9 +18,10 @@ struct Geom {
 // when the lattice is wide enough; BX divides nx when possible so no lane
 // idles.
 Geom make_geom(int nx, int ny, int nz, int threads = 256);
-// the same for a step that sums nothing: blocks of consecutive nodes where rows
-// are no multiple of 32
-Geom make_step_geom(int nx, int ny, int nz);
+// the same for a step that sums nothing, of q populations in arithmetic of `real`
+// bytes: blocks of consecutive nodes where rows are no multiple of 32 and the
+// lattice is large enough
+Geom make_step_geom(int nx, int ny, int nz, int q, size_t real);
 
 struct FlowLaunch {
     const void* fin;

@@ -21,8 +21,16 @@ Geom make_geom(int nx, int ny, int nz, int threads) {
     return g;
 }
 
-Geom make_step_geom(int nx, int ny, int nz) {
-    if (nx % 32 == 0) return make_geom(nx, ny, nz);
+Geom make_step_geom(int nx, int ny, int nz, int q, size_t real) {
+    // nodes from which on consecutive nodes won at every width tried (24 to 330;
+    // below, the two are within 5 % or differ either way with the shape: dividing
+    // for the coordinates costs about 0.1 us, and lattices this small are bound by
+    // latency).  Temperature step, us: 200 x 33 x 33 3.13 in tiles, 3.52; 200 x 40 x 40
+    // 3.81, 3.65.  Flow forward: 48 x 50 x 50 4.15, 4.45; 147 x 33 x 33 5.17, 4.32.  2D
+    // FP32: 1000 x 1000 9.50, 10.07; 1501 x 1200 26.4, 25.5.  64-bit arithmetic loses
+    // most to idle lanes: 48 x 41 x 41 35.2, 28.4; 24 x 13 x 13 16.7, 20.0.
+    const long long least = real == 8 ? 50000 : (q == 19 ? 150000 : (q == 7 ? 250000 : 1200000));
+    if (nx % 32 == 0 || (long long)nx * ny * nz < least) return make_geom(nx, ny, nz);
     Geom g;
     g.block = dim3(256, 1, 1);
     g.grid = dim3((unsigned)(((long long)nx * ny * nz + 255) / 256), 1, 1);

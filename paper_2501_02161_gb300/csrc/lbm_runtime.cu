@@ -101,7 +101,7 @@ struct lbm_ctx {
     long long launches = 0;  // kernels launched (lbm_launches)
 
     Geom geom{};
-    Geom step_geom{};  // of the plain steps
+    Geom step_geom{}, heat_geom{};  // of the plain steps: flow, temperature
     lbm_params prm{0.6, 1.0, 0, 0.0, 1.0, 0.0, 0.0, 0.0};
     lbm_objective obj{1.0, 0.0, 0.0};
     long long n_in = 0, n_nw = 0;
@@ -238,7 +238,8 @@ cudaError_t enqueue_step(lbm_ctx* c, int ph, bool reduce, cudaStream_t s, bool a
     cudaError_t e = cudaSuccess;
     const int* bail = after_resident ? (const int*)(c->sync + 1) : nullptr;
     const bool cont = ph == PH_ADJ && c->adj_scheme == LBM_ADJOINT_CONTINUOUS;  // keeps the tiles
-    const Geom& geom = reduce || cont ? c->geom : c->step_geom;
+    const bool heat = ph == PH_THERM || ph == PH_TADJ;
+    const Geom& geom = reduce || cont ? c->geom : (heat ? c->heat_geom : c->step_geom);
     if (ph == PH_FLOW) {
         FlowLaunch a = flow_base(c);
         a.fin = c->f[c->fcur];
@@ -836,7 +837,8 @@ lbm_status lbm_create(lbm_ctx** out, int stencil, int nx, int ny, int nz, int st
     c->ab = adj_bytes(storage);
     c->rb = aux_bytes(storage);
     c->geom = make_geom(nx, ny, nz);
-    c->step_geom = make_step_geom(nx, ny, nz);
+    c->step_geom = make_step_geom(nx, ny, nz, c->Q, c->rb);
+    c->heat_geom = make_step_geom(nx, ny, nz, 7, c->rb);
     c->inbox_bytes = resident_plans(stencil, nx, ny, nz, storage, c->thermal, c->plan);
     cudaError_t e = cudaSuccess;
     e = cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking);
