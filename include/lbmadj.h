@@ -373,7 +373,10 @@ lbm_status lbm_import_state(lbm_ctx* ctx, const void* src, size_t bytes);
 typedef struct lbm_batch lbm_batch;
 
 /* Bytes of device memory lbm_create allocates for a context of this shape
- * (for admission by HBM footprint). */
+ * (for admission by HBM footprint).  The first solve of its own (lbm_forward and
+ * the like, not a batch's steps) of a lattice that fits on the chip allocates some
+ * megabytes more for its resident launches (64^3 FP32: 7.7 beside 90), or does
+ * without them. */
 size_t lbm_footprint_bytes(int stencil, int nx, int ny, int nz, int storage, int thermal);
 
 /* storage: the storage every admitted context must use; check_every: K, even,

@@ -89,15 +89,16 @@ struct lbm_ctx {
     double* partials = nullptr;
     double* dres = nullptr;
     double* hres = nullptr;  // pinned, 4 doubles
-    ResPlan plan[4] = {};    // per phase: how its lattice is cut for a resident launch
-    void* inbox = nullptr;   // words exchanged by resident launches
-    unsigned* sync = nullptr;  // their step counter and error flag
+    // resident launches, set up by the first block that may be one (prepare_resident)
+    bool prepared = false;
+    ResPlan plan[4] = {};    // per phase: how its lattice is cut (ok: it fits on the chip)
+    void* inbox = nullptr;   // the words they exchange
     size_t inbox_bytes = 0;
+    unsigned* sync = nullptr;  // their step counter and error flag
     unsigned long long tags = 0;  // step numbers used since the counter was cleared
     int min_steps = 0;       // plain steps that go resident (0: resident_min_steps)
     int wait_limit = kWaitLimit;  // polls after which a resident launch gives up waiting
-    bool resident = false;
-    int gave_up = 0;         // resident launches that were refused or gave up waiting
+    int gave_up = 0;         // resident launches that were refused, gave up waiting or found no memory
     long long launches = 0;  // kernels launched (lbm_launches)
 
     Geom geom{};
@@ -129,20 +130,6 @@ struct lbm_ctx {
 namespace {
 // a destroyed context stops counting against its batch's memory budget
 void batch_forget(lbm_batch* b, lbm_ctx* c);
-
-// the cuts of a lattice's phases (out: PH_* order) and the bytes their inboxes need
-size_t resident_plans(int stencil, int nx, int ny, int nz, int storage, bool thermal, ResPlan (&out)[4]) {
-    out[PH_FLOW] = resident_plan(stencil, storage, RP_FLOW, nx, ny, nz);
-    out[PH_ADJ] = resident_plan(stencil, storage, thermal ? RP_ADJ_T : RP_ADJ, nx, ny, nz);
-    if (thermal) {
-        out[PH_THERM] = resident_plan(stencil, storage, RP_THERM, nx, ny, nz);
-        out[PH_TADJ] = resident_plan(stencil, storage, RP_TADJ, nx, ny, nz);
-    }
-    size_t bytes = 0;
-    for (const ResPlan& p : out)
-        if (p.ok) bytes = std::max(bytes, p.inbox_bytes);
-    return bytes;
-}
 
 void* dalloc(size_t bytes, cudaError_t* err) {
     void* p = nullptr;
@@ -308,10 +295,49 @@ int resident_min_steps(const lbm_ctx* c, int ph) {
 // launch per step.
 constexpr int kResidentTries = 3;
 
-bool resident_fits(const lbm_ctx* c, int ph, int steps) {
-    return c->resident && c->gave_up < kResidentTries && c->plan[ph].ok &&
-           steps >= resident_min_steps(c, ph) &&
-           !(ph == PH_ADJ && c->adj_scheme == LBM_ADJOINT_CONTINUOUS);
+// The cuts of a context's phases (40 to 180 us of host time) and its inboxes (0.3
+// to 12.4 MB; 64^3 FP32: 7.7 beside 90): made for the first block that
+// may go resident, so that a context of a batch, which never does, neither waits
+// nor pays for them.  Without memory for the inboxes the context steps by
+// launches.
+void prepare_resident(lbm_ctx* c) {
+    c->prepared = true;
+    int sms = 0, coop = 0, smem = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c->device);
+    cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
+    const ResPhase phases[4] = {RP_FLOW, RP_THERM, c->thermal ? RP_ADJ_T : RP_ADJ, RP_TADJ};
+    for (int ph = 0; ph < 4; ++ph) {
+        if (!c->thermal && (ph == PH_THERM || ph == PH_TADJ)) continue;
+        ResPlan p = resident_plan(c->stencil, c->storage, phases[ph], c->nx, c->ny, c->nz);
+        p.ok = p.ok && coop && sms * p.per_sm >= p.g.px * p.g.py * p.g.pz && (size_t)smem >= p.smem;
+        if (p.ok) c->inbox_bytes = std::max(c->inbox_bytes, p.inbox_bytes);
+        c->plan[ph] = p;
+    }
+    if (!c->inbox_bytes) return;
+    // (an allocation of this thread has no part in what another one captures)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    cudaError_t e = cudaSuccess;
+    c->inbox = dalloc(c->inbox_bytes, &e);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->inbox, 0, c->inbox_bytes, c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->sync, 0, 2 * sizeof(unsigned), c->stream);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        if (c->inbox) cudaFree(c->inbox);
+        c->inbox = nullptr;
+        c->prepared = false;
+        ++c->gave_up;
+    }
+}
+
+bool resident_fits(lbm_ctx* c, int ph, int steps) {
+    if (c->gave_up >= kResidentTries || steps < resident_min_steps(c, ph)) return false;
+    if (ph == PH_ADJ && c->adj_scheme == LBM_ADJOINT_CONTINUOUS) return false;
+    if (!c->prepared) prepare_resident(c);
+    if (!c->prepared) return false;
+    return c->plan[ph].ok && steps >= resident_min_steps(c, ph);  // (it may ask the plan)
 }
 
 // enqueue n plain steps of a phase as one resident launch
@@ -839,7 +865,6 @@ lbm_status lbm_create(lbm_ctx** out, int stencil, int nx, int ny, int nz, int st
     c->geom = make_geom(nx, ny, nz);
     c->step_geom = make_step_geom(nx, ny, nz, c->Q, c->rb);
     c->heat_geom = make_step_geom(nx, ny, nz, 7, c->rb);
-    c->inbox_bytes = resident_plans(stencil, nx, ny, nz, storage, c->thermal, c->plan);
     cudaError_t e = cudaSuccess;
     e = cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev, cudaEventDisableTiming);
@@ -872,23 +897,11 @@ lbm_status lbm_create(lbm_ctx** out, int stencil, int nx, int ny, int nz, int st
     }
     c->partials = (double*)dalloc(sizeof(double) * 2 * (size_t)c->geom.nblocks, &e);
     c->dres = (double*)dalloc(sizeof(double) * 4 + 2 * sizeof(unsigned), &e);
-    if (c->inbox_bytes) c->inbox = dalloc(c->inbox_bytes, &e);
     if (c->dres) c->sync = (unsigned*)(c->dres + 4);
     if (e == cudaSuccess) e = cudaMallocHost(&c->hres, sizeof(double) * 4);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->flags, 1 /* WALL */, np, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->bc, 0, np * 4 * c->rb, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->gamma, 0, np * c->rb, c->stream);
-    if (e == cudaSuccess && c->inbox_bytes) {
-        e = cudaMemsetAsync(c->inbox, 0, c->inbox_bytes, c->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(c->sync, 0, 2 * sizeof(unsigned), c->stream);
-        int sms = 0, coop = 0, smem = 0;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c->device);
-        cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
-        c->resident = coop != 0;
-        for (const ResPlan& p : c->plan)
-            if (p.ok) c->resident &= sms * p.per_sm >= p.g.px * p.g.py * p.g.pz && (size_t)smem >= p.smem;
-    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
         free_all(c);
@@ -1345,9 +1358,10 @@ lbm_status lbm_set_resident(lbm_ctx* c, int min_steps, int wait_limit, unsigned 
     if (!c) return fail(LBM_ERR_ARG, "ctx is null");
     if (min_steps < 0 || wait_limit < 0) return fail(LBM_ERR_ARG, "negative argument");
     c->min_steps = min_steps;
-    if (!c->inbox) return LBM_OK;
     lbm_status st = enter(c);
     if (st != LBM_OK) return st;
+    if (!c->prepared) prepare_resident(c);
+    if (!c->inbox) return leave(c);
     const unsigned sync[2] = {step_number, 0};
     CUDA_TRY(cudaMemsetAsync(c->inbox, 0, c->inbox_bytes, c->stream));
     CUDA_TRY(cudaMemcpyAsync(c->sync, sync, sizeof(sync), cudaMemcpyHostToDevice, c->stream));
@@ -1710,8 +1724,6 @@ size_t lbm_footprint_bytes(int stencil, int nx, int ny, int nz, int storage, int
     if (thermal) bytes += 2 * np * 7 * (hb + ab) + np * rb * (1 + 7 + 3 + 1 + 1);
     Geom g = make_geom(nx, ny, nz);
     bytes += sizeof(double) * 2 * (size_t)g.nblocks + 64;
-    ResPlan plans[4] = {};
-    bytes += resident_plans(stencil, nx, ny, nz, storage, thermal != 0, plans);
     return bytes;
 }
 
