@@ -310,6 +310,11 @@ lbm_status lbm_time_steps(lbm_ctx* ctx, int phase, int n, double* ms_per_step);
  * inputs and outputs, lbm_time_steps and packed batch launches are not counted. */
 long long lbm_launches(lbm_ctx* ctx);
 
+/* Phases (bit p: phase p of lbm_solve_phase) whose lattice fits on the chip, so
+ * that blocks of enough plain steps go resident; 0 for a lattice lbm_create
+ * refuses.  A host function. */
+int lbm_resident_phases(int stencil, int nx, int ny, int nz, int storage, int thermal);
+
 /* When the context's plain steps go resident, and how such launches wait and
  * count (no effect on a lattice that has none): min_steps, the plain steps of a
  * block from which on they are one resident launch (by default 0: where that
@@ -488,7 +493,8 @@ const char* lbm_last_error(void);
  * how many computed sources differ from the periodic wrap of x -/+ e_i or fall
  * outside the lattice.  For a lattice small enough for resident launches the
  * count includes the populations that such a launch would send to another word
- * than their receiver reads, under every set of symmetry planes.  stencil: 0 D2Q9, 1 D3Q19, 2 D3Q7 (temperature).
+ * than their receiver reads, in every phase and storage that fits on the chip
+ * and under every set of symmetry planes.  stencil: 0 D2Q9, 1 D3Q19, 2 D3Q7 (temperature).
  * Errors: LBM_ERR_ARG (null pointer, bad sizes, more than 2^24 nodes). */
 lbm_status lbm_check_addressing(int stencil, int nx, int ny, int nz, long long* mismatches);
 

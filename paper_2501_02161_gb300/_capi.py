@@ -93,6 +93,7 @@ SIGNATURES = {
     "lbm_get_adjoint": (_I, [_VP, _VP, _VP, _I, _I]),
     "lbm_time_steps": (_I, [_VP, _I, _I, ctypes.POINTER(ctypes.c_double)]),
     "lbm_launches": (ctypes.c_longlong, [_VP]),
+    "lbm_resident_phases": (_I, [_I, _I, _I, _I, _I, _I]),
     "lbm_set_resident": (_I, [_VP, _I, _I, ctypes.c_uint]),
     "lbm_flow_step_noalloc": (_I, [ctypes.POINTER(lbm_step_desc), _VP]),
     "lbm_footprint_bytes": (ctypes.c_size_t, [_I, _I, _I, _I, _I, _I]),

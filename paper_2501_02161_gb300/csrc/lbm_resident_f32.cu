@@ -127,7 +127,7 @@ namespace {
 // it from, inside the inboxes and used once; and every word that is waited for
 // has to be sent.
 template <class P>
-long long exchange_mismatches(const ResGeom& g, int mirror) {
+long long exchange_mismatches(const ResGeom& g, int mirror, std::vector<long long>& leaves) {
     using L = typename P::L;
     constexpr int NP = res_per_word<P>();
     const int dim[3] = {g.nx, g.ny, g.nz};
@@ -186,7 +186,12 @@ long long exchange_mismatches(const ResGeom& g, int mirror) {
                     }
                 }
             }
-            // the items are all (node, population) pairs that leave; the others stay in the box
+            // the items are all (node, population) pairs that leave (whatever the
+            // symmetry planes); the others stay in the box
+            if (mirror || pass) {
+                bad += items != leaves[blk];
+                continue;
+            }
             long long leaving = 0;
             for (int lz = 0; lz < b.ez; ++lz)
                 for (int ly = 0; ly < b.ey; ++ly)
@@ -201,37 +206,55 @@ long long exchange_mismatches(const ResGeom& g, int mirror) {
                                             res_move<P>(i, 2) * b.sz;
                             bad += far < 0 || far >= g.cap;
                         }
+            leaves[blk] = leaving;
             bad += items != leaving;
         }
     for (int w : waits) bad += w;
     return bad + (sent != read);
 }
 
+// the exchange is the same for phases of equal cuts whose populations move the
+// same way, as one or three to a word
+struct Checked {
+    ResGeom g;
+    int way, per_word;
+};
+
 template <class P>
-long long exchange_check(int stencil, int storage, ResPhase ph, int nx, int ny, int nz) {
+long long exchange_check(int stencil, int storage, ResPhase ph, int nx, int ny, int nz, std::vector<Checked>& done) {
     const ResPlan p = resident_plan(stencil, storage, ph, nx, ny, nz);
     if (!p.ok) return 0;
+    for (const Checked& d : done)
+        if (d.way == P::S && d.per_word == res_per_word<P>() && d.g.bx == p.g.bx && d.g.by == p.g.by &&
+            d.g.bz == p.g.bz && d.g.cap == p.g.cap && d.g.inbox == p.g.inbox)
+            return 0;
+    done.push_back({p.g, P::S, res_per_word<P>()});
     long long bad = 0;
-    for (int mirror = 0; mirror < (stencil == 0 ? 4 : 8); ++mirror) bad += exchange_mismatches<P>(p.g, mirror);
+    std::vector<long long> leaves((size_t)p.g.px * p.g.py * p.g.pz);
+    for (int mirror = 0; mirror < (stencil == 0 ? 4 : 8); ++mirror) bad += exchange_mismatches<P>(p.g, mirror, leaves);
     return bad;
 }
 
+// every phase that a context of one storage can have
 template <typename R>
-long long exchange_checks(int stencil, int nx, int ny, int nz) {
-    const int st = sizeof(R) == 8 ? 0 : 1;
-    if (stencil == 0)
-        return exchange_check<ResFlow<D2Q9, R, R, R>>(0, st, RP_FLOW, nx, ny, nz) +
-               exchange_check<ResAdjoint<D2Q9, R, R, false>>(0, st, RP_ADJ, nx, ny, nz);
+long long exchange_checks(int stencil, int storage, int nx, int ny, int nz, std::vector<Checked>& done) {
+    auto check = [&](auto phase, ResPhase ph) {
+        return exchange_check<decltype(phase)>(stencil == 0 ? 0 : 1, storage, ph, nx, ny, nz, done);
+    };
+    if (stencil == 0) return check(ResFlow<D2Q9, R, R, R>(), RP_FLOW) + check(ResAdjoint<D2Q9, R, R, false>(), RP_ADJ);
     if (stencil == 1)
-        return exchange_check<ResFlow<D3Q19, R, R, R>>(1, st, RP_FLOW, nx, ny, nz) +
-               exchange_check<ResAdjoint<D3Q19, R, R, true>>(1, st, RP_ADJ_T, nx, ny, nz);
-    return exchange_check<ResHeat<R, R, R>>(1, st, RP_THERM, nx, ny, nz) +
-           exchange_check<ResHeatAdjoint<R, R>>(1, st, RP_TADJ, nx, ny, nz);
+        return check(ResFlow<D3Q19, R, R, R>(), RP_FLOW) + check(ResAdjoint<D3Q19, R, R, false>(), RP_ADJ) +
+               check(ResAdjoint<D3Q19, R, R, true>(), RP_ADJ_T);
+    return check(ResHeat<R, R, R>(), RP_THERM) + check(ResHeatAdjoint<R, R>(), RP_TADJ);
 }
 }  // namespace
 
 long long resident_mismatches(int stencil, int nx, int ny, int nz) {
-    return exchange_checks<float>(stencil, nx, ny, nz) + exchange_checks<double>(stencil, nx, ny, nz);
+    std::vector<Checked> done;
+    long long bad = exchange_checks<double>(stencil, 0, nx, ny, nz, done);
+    for (int storage = 1; storage < (stencil == 0 ? 2 : 4); ++storage)
+        bad += exchange_checks<float>(stencil, storage, nx, ny, nz, done);
+    return bad;
 }
 
 cudaError_t resident_flow_f64(int stencil, ResPhase ph, const FlowLaunch& a, const ResPlan& p, const ResWords& w,

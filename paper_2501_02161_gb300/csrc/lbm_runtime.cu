@@ -295,6 +295,13 @@ int resident_min_steps(const lbm_ctx* c, int ph) {
 // launch per step.
 constexpr int kResidentTries = 3;
 
+// how a phase's lattice is cut
+ResPlan phase_plan(int stencil, int nx, int ny, int nz, int storage, bool thermal, int ph) {
+    const ResPhase phases[4] = {RP_FLOW, RP_THERM, thermal ? RP_ADJ_T : RP_ADJ, RP_TADJ};
+    if (!thermal && (ph == PH_THERM || ph == PH_TADJ)) return ResPlan{};
+    return resident_plan(stencil, storage, phases[ph], nx, ny, nz);
+}
+
 // The cuts of a context's phases (40 to 180 us of host time) and its inboxes (0.3
 // to 12.4 MB; 64^3 FP32: 7.7 beside 90): made for the first block that
 // may go resident, so that a context of a batch, which never does, neither waits
@@ -306,10 +313,8 @@ void prepare_resident(lbm_ctx* c) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c->device);
     cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
-    const ResPhase phases[4] = {RP_FLOW, RP_THERM, c->thermal ? RP_ADJ_T : RP_ADJ, RP_TADJ};
     for (int ph = 0; ph < 4; ++ph) {
-        if (!c->thermal && (ph == PH_THERM || ph == PH_TADJ)) continue;
-        ResPlan p = resident_plan(c->stencil, c->storage, phases[ph], c->nx, c->ny, c->nz);
+        ResPlan p = phase_plan(c->stencil, c->nx, c->ny, c->nz, c->storage, c->thermal, ph);
         p.ok = p.ok && coop && sms * p.per_sm >= p.g.px * p.g.py * p.g.pz && (size_t)smem >= p.smem;
         if (p.ok) c->inbox_bytes = std::max(c->inbox_bytes, p.inbox_bytes);
         c->plan[ph] = p;
@@ -836,6 +841,16 @@ lbm_status lbm_check_addressing(int stencil, int nx, int ny, int nz, long long* 
 }
 
 const char* lbm_version(void) { return "lbmadj 0.1 (sm_103a)"; }
+
+int lbm_resident_phases(int stencil, int nx, int ny, int nz, int storage, int thermal) {
+    if (stencil != LBM_D2Q9 && stencil != LBM_D3Q19) return 0;
+    if (storage < LBM_FP64 || storage > LBM_BF16_OFS || nx <= 0 || ny <= 0 || nz <= 0) return 0;
+    if (stencil == LBM_D2Q9 && (nz != 1 || thermal || storage > LBM_FP32)) return 0;
+    int mask = 0;
+    for (int ph = 0; ph < 4; ++ph)
+        mask |= (int)phase_plan(stencil, nx, ny, nz, storage, thermal != 0, ph).ok << ph;
+    return mask;
+}
 
 lbm_status lbm_create(lbm_ctx** out, int stencil, int nx, int ny, int nz, int storage, int thermal) {
     if (!out) return fail(LBM_ERR_ARG, "out is null");
