@@ -495,7 +495,8 @@ const char* lbm_last_error(void);
  * count includes the populations that such a launch would send to another word
  * than their receiver reads, in every phase and storage that fits on the chip
  * and under every set of symmetry planes.  stencil: 0 D2Q9, 1 D3Q19, 2 D3Q7 (temperature).
- * Errors: LBM_ERR_ARG (null pointer, bad sizes, more than 2^24 nodes). */
+ * Errors: LBM_ERR_ARG (null pointer, bad sizes, more than 2^24 nodes),
+ * LBM_ERR_OOM (host memory). */
 lbm_status lbm_check_addressing(int stencil, int nx, int ny, int nz, long long* mismatches);
 
 const char* lbm_version(void);

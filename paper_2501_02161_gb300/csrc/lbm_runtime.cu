@@ -19,6 +19,7 @@
 #include <atomic>
 #include <map>
 #include <mutex>
+#include <new>
 #include <shared_mutex>
 #include <string>
 #include <tuple>
@@ -836,7 +837,11 @@ lbm_status lbm_check_addressing(int stencil, int nx, int ny, int nz, long long* 
     if (stencil < 0 || stencil > 2) return fail(LBM_ERR_ARG, "unknown stencil");
     if (nx <= 0 || ny <= 0 || nz <= 0) return fail(LBM_ERR_ARG, "lattice sizes must be positive");
     if ((long long)nx * ny * nz > (1LL << 24)) return fail(LBM_ERR_ARG, "at most 2^24 nodes (a host loop)");
-    *mismatches = addressing_mismatches(stencil, nx, ny, nz) + resident_mismatches(stencil, nx, ny, nz);
+    try {
+        *mismatches = addressing_mismatches(stencil, nx, ny, nz) + resident_mismatches(stencil, nx, ny, nz);
+    } catch (const std::bad_alloc&) {
+        return fail(LBM_ERR_OOM, "host memory for the check");
+    }
     return LBM_OK;
 }
 

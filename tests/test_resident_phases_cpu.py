@@ -6,6 +6,9 @@ temperature, flow adjoint, temperature adjoint), so that a phase that silently
 loses its cut, and its check with it, is seen.
 """
 import ctypes
+import os
+import subprocess
+import sys
 
 import pytest
 
@@ -61,3 +64,20 @@ def test_lattices_that_are_refused_have_no_phases():
     phases = C.lib().lbm_resident_phases
     assert phases(0, 64, 64, 2, 1, 0) == phases(0, 64, 64, 1, 2, 0) == phases(0, 64, 64, 1, 1, 1) == 0
     assert phases(1, 0, 16, 16, 1, 0) == phases(1, 16, 16, 16, 4, 0) == phases(2, 16, 16, 16, 1, 0) == 0
+
+
+def test_no_host_memory_is_an_error_not_an_abort():
+    """The check's tables do not fit under the limit set here; the call reports it."""
+    code = """
+import ctypes, resource, sys
+sys.path.insert(0, {root!r})
+from paper_2501_02161_gb300 import _capi as C
+L = C.lib()
+vm = int(open("/proc/self/statm").read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (vm + (1 << 20), vm + (1 << 20)))
+bad = ctypes.c_longlong(-1)
+sys.exit(0 if L.lbm_check_addressing(1, 64, 64, 64, ctypes.byref(bad)) == C.LBM_ERR_OOM else 3)
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", code.format(root=root)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
