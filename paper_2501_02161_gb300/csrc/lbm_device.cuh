@@ -919,7 +919,8 @@ __device__ __forceinline__ void pull_adjoint(const FlowArgs<T, TA, R>& a, const 
 
 // resident 256-thread blocks per SM requested from the compiler: the plain
 // FP32-math D3Q19 adjoint fits 40 registers without spilling (6 blocks, 75 %
-// occupancy), its thermal-coupling variant 48 (5 blocks); the reducing
+// occupancy; with symmetry planes it spills 24 bytes), its thermal-coupling
+// variant 48 (5 blocks); the reducing
 // variants (one step in K) keep the compiler's choice; the plain adjoint over
 // consecutive nodes takes 48 (8 bytes would spill at 40)
 template <class L, typename R, bool REDUCE, bool THERMAL>
@@ -933,15 +934,16 @@ struct AdjMinBlocks {
 // adjoint collision at a non-wall node, in place (Eq. 63-65): f*_C,i =
 // (1 - 1/tau) f*_S,i + (1/tau) sum_m (d f^eq_m / d f_i) f*_S,m
 // [- dJ/df_i = 1/(3 N_in) at an inlet node when src] [+ thermal coupling]
-// Taking its operands as values lets the coupled step read them ahead of the
-// moments (320 x 160 x 80: 18.9 against 19.3 ms a pass, 192 x 96 x 48 11.7 against
-// 12.0); the plain step spills 4 bytes for it (256^3 40.95 against 40.86 ms).
-template <class L, typename R>
-__device__ __forceinline__ void adjoint_collide_values(R om, int model, R src_in, bool src, R g, R u0, R u1, R u2,
-                                                       R v0, R v1, R v2, R (&s)[L::Q]) {
+// take(g, u, v) gives the operands (gamma, velocity, coupling) after the moments
+template <class L, typename R, class Take>
+__device__ __forceinline__ void adjoint_collide_with(const R& omega, const int& model, const R& src_in, bool src,
+                                                     Take take, R (&s)[L::Q]) {
     using X = Ex<R>;
     AdjMoments<L, R> m;
     m.compute(s);
+    R g, u[3], v[3] = {0, 0, 0};
+    take(g, u, v);
+    const R om = omega, u0 = u[0], u1 = u[1], u2 = u[2], v0 = v[0], v1 = v[1], v2 = v[2];
     const R Qu0 = X::fma(m.Q02, u2, X::fma(m.Q01, u1, X::mul(m.Q00, u0)));
     const R Qu1 = X::fma(m.Q12, u2, X::fma(m.Q11, u1, X::mul(m.Q01, u0)));
     const R Qu2 = X::fma(m.Q22, u2, X::fma(m.Q12, u1, X::mul(m.Q02, u0)));
@@ -972,16 +974,37 @@ __device__ __forceinline__ void adjoint_collide_values(R om, int model, R src_in
     }
 }
 
+// the same with its operands as values
+template <class L, typename R>
+__device__ __forceinline__ void adjoint_collide_values(R om, int model, R src_in, bool src, R g0, R u0, R u1, R u2,
+                                                       R v0, R v1, R v2, R (&s)[L::Q]) {
+    adjoint_collide_with<L, R>(om, model, src_in, src,
+                               [&](R& g, R (&u)[3], R (&v)[3]) {
+                                   g = g0;
+                                   u[0] = u0; u[1] = u1; u[2] = u2;
+                                   v[0] = v0; v[1] = v1; v[2] = v2;
+                               },
+                               s);
+}
+
+// The coupled step gains by reading its operands ahead of the moments
+// (320 x 160 x 80: 109.3 against 115.2 us a step); at the plain step's 40 registers
+// that would spill (256^3: 406.5 against 404.9 us).
 template <class L, typename T, typename TA, typename R, bool THERMAL, bool CPL_RT>
 __device__ __forceinline__ void adjoint_collide(const FlowArgs<T, TA, R>& a, long long n, bool src, R (&s)[L::Q]) {
-    R v0 = 0, v1 = 0, v2 = 0;
-    if (THERMAL || (CPL_RT && a.cpl != nullptr)) {
-        v0 = a.cpl[n];
-        v1 = a.cpl[a.np + n];
-        v2 = a.cpl[2 * a.np + n];
+    if constexpr (THERMAL) {
+        adjoint_collide_values<L, R>(a.omega, a.model, a.src_in, src, a.gamma[n], a.u[n], a.u[a.np + n],
+                                     a.u[2 * a.np + n], a.cpl[n], a.cpl[a.np + n], a.cpl[2 * a.np + n], s);
+    } else {
+        adjoint_collide_with<L, R>(a.omega, a.model, a.src_in, src,
+                                   [&](R& g, R (&u)[3], R (&v)[3]) {
+                                       g = a.gamma[n];
+                                       for (int k = 0; k < 3; ++k) u[k] = a.u[k * a.np + n];
+                                       if (CPL_RT && a.cpl != nullptr)
+                                           for (int k = 0; k < 3; ++k) v[k] = a.cpl[k * a.np + n];
+                                   },
+                                   s);
     }
-    adjoint_collide_values<L, R>(a.omega, a.model, a.src_in, src, a.gamma[n], a.u[n], a.u[a.np + n],
-                                 a.u[2 * a.np + n], v0, v1, v2, s);
 }
 
 template <class L, typename T, typename TA, typename R, bool REDUCE, bool THERMAL, bool CPL_RT = false,
