@@ -665,8 +665,8 @@ def run_ours(args):
     # kernel time shares inside the workload: per-launch duration at 64^3
     s0 = solvers[RES[1]]
     s0.forward(tol=0, max_steps=2, check_every=2, reset=True)
-    fwd_ms_w = s0.time_steps(0, 200)
-    adj_ms_w = s0.time_steps(2, 200)
+    fwd_ms_w = s0.time_steps(0, 2 * CHECK)  # two blocks of a solve
+    adj_ms_w = s0.time_steps(2, 2 * CHECK)
     fsteps = sum(v["fwd_steps"] for v in per.values())
     asteps = sum(v["adj_steps"] for v in per.values())
     fwd_share = fsteps * fwd_ms_w / (fsteps * fwd_ms_w + asteps * adj_ms_w)

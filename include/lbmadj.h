@@ -293,8 +293,8 @@ lbm_status lbm_get_objective(lbm_ctx* ctx, double* J);
 lbm_status lbm_get_adjoint(lbm_ctx* ctx, void* fstar, void* gstar, int dtype, int on_device);
 
 /* Time plain steps of one phase as a solve runs them (a launch each, or two
- * resident launches with a step of its own after each when the lattice fits on
- * the chip): n steps (rounded up to even) are captured as a CUDA graph, replayed
+ * resident launches with a step of its own after each, when the lattice fits on
+ * the chip and n / 2 steps are enough for one): n steps (rounded up to even) are captured as a CUDA graph, replayed
  * once untimed, then replayed between two CUDA events recorded on the context's
  * stream; writes the mean milliseconds per step of the timed replay (kernel
  * time plus the gaps between graph nodes).  phase: 0 flow forward, 1

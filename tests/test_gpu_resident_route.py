@@ -14,6 +14,7 @@ torch = pytest.importorskip("torch")
 
 from paper_2501_02161_gb300 import _capi as C
 from paper_2501_02161_gb300 import inputs as I
+from test_gpu_resident import CASES, LATTICES as LATTICES_OF_ALL_KINDS
 
 pytestmark = pytest.mark.gpu
 
@@ -256,3 +257,35 @@ def test_resident_launches_of_few_steps(name, storage, check):
     # initial populations (the temperature's also collide), blocks, coupling, dJ/dgamma
     assert s.launches() - n == phases + 2 * (phases == 4) + phases * -(-60 // check) * 3 + 1
     s.close()
+
+
+@pytest.mark.parametrize("name,storage", CASES, ids=lambda v: v)
+def test_every_phase_with_a_cut_goes_resident(name, storage):
+    """One box and many, cut boxes, axes of length 1 to 3, symmetry planes, all
+    kinds of openings, every storage: the phases that fit on the chip, and only
+    they, take 3 launches a block, and the results are those of single steps."""
+    lat = LATTICES_OF_ALL_KINDS[name]()
+    for steps in (13, 50):
+        s = solver(lat, storage)
+        ref = solve(s, steps, 1)
+        set_resident(s, min_steps=1)
+        n = s.launches()
+        same(solve(s, steps, steps), ref)
+        code = {"fp64": 0, "fp32": 1, "fp16": 2, "bf16": 3}[storage]
+        fits = s.lib.lbm_resident_phases(lat.stencil, lat.nx, lat.ny, lat.nz, code, int(s.thermal))
+        phases = (0, 1, 2, 3) if s.thermal else (0, 2)
+        blocks = sum(3 if fits >> p & 1 else steps + 1 for p in phases)
+        assert fits and s.launches() - n == len(phases) + 2 * s.thermal + blocks + 1
+        s.close()
+
+
+def test_contexts_of_different_sizes_in_turn():
+    """Each size asks for its own shared memory; a captured launch of the larger
+    one still runs resident after the smaller one's."""
+    a, b = solver(I.pipe_bend_3d(64, width=16, re=20.0, seed=2)), solver(I.pipe_bend_3d(16, width=4, re=10.0, seed=2))
+    for s in (a, b, a, b, a):
+        n = s.launches()
+        s.forward(tol=0, max_steps=400, check_every=100)
+        assert s.launches() - n == 1 + 4 * 3
+    a.close()
+    b.close()
