@@ -294,13 +294,14 @@ lbm_status lbm_get_adjoint(lbm_ctx* ctx, void* fstar, void* gstar, int dtype, in
 
 /* Time plain steps of one phase as a solve runs them (a launch each, or two
  * resident launches with a step of its own after each, when the lattice fits on
- * the chip and n / 2 steps are enough for one): n steps (rounded up to even) are captured as a CUDA graph, replayed
- * once untimed, then replayed between two CUDA events recorded on the context's
- * stream; writes the mean milliseconds per step of the timed replay (kernel
- * time plus the gaps between graph nodes).  phase: 0 flow forward, 1
- * temperature forward, 2 flow adjoint, 3 temperature adjoint.  The 2n steps
- * advance that phase's state as a solve would; no reduction runs.  Needs the inputs set (LBM_ERR_ORDER) and, for
- * phases 1-3, a completed lbm_forward.  After LBM_ERR_CUDA from a wait that gave
+ * the chip and n / 2 steps are enough for one): n steps (rounded up to even) are
+ * captured as a CUDA graph, replayed once untimed, then replayed between two
+ * CUDA events recorded on the context's stream; writes the mean milliseconds
+ * per step of the timed replay (kernel time plus the gaps between graph nodes).
+ * phase: 0 flow forward, 1 temperature forward, 2 flow adjoint, 3 temperature
+ * adjoint.  The 2n steps advance that phase's state as a solve would; no
+ * reduction runs.  Needs the inputs set (LBM_ERR_ORDER) and, for phases 1-3, a
+ * completed lbm_forward.  After LBM_ERR_CUDA from a wait that gave
  * up, the phase and those after it have to be solved again. */
 lbm_status lbm_time_steps(lbm_ctx* ctx, int phase, int n, double* ms_per_step);
 

@@ -463,6 +463,9 @@ lbm_status run_block(lbm_ctx* c, int ph, int k, bool resident) {
 lbm_status run_block_sync(lbm_ctx* c, int ph, int k, const InFlight& solve) {
     std::shared_mutex& chip = g_chip[c->device & 63];
     if (resident_fits(c, ph, k - 1) && solve.alone()) {
+        // what the caller's stream holds comes first, without the lock: it may
+        // take long, or wait for what another thread does
+        CUDA_TRY(cudaEventSynchronize(c->ev));
         std::unique_lock<std::shared_mutex> lock(chip);
         if (run_block(c, ph, k, true) == LBM_OK) {
             CUDA_TRY(cudaStreamSynchronize(c->stream));
@@ -1491,6 +1494,7 @@ lbm_status lbm_time_steps(lbm_ctx* c, int phase, int n, double* ms_per_step) {
     // (the step numbers of all replays stay below the restart's threshold)
     const bool resident = m <= 1 << 28 && resident_fits(c, phase, (int)(m / 2) - 1) && solve.alone();
     if (resident) {
+        CUDA_TRY(cudaEventSynchronize(c->ev));
         std::unique_lock<std::shared_mutex> lock(g_chip[c->device & 63]);
         st = time_replay(c, phase, m, true, &began, &ms);
         if (st != LBM_OK && !began) {  // refused: nothing has run

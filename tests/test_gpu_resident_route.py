@@ -289,3 +289,28 @@ def test_contexts_of_different_sizes_in_turn():
         assert s.launches() - n == 1 + 4 * 3
     a.close()
     b.close()
+
+
+def test_a_solve_that_waits_for_its_stream_holds_up_no_other():
+    """A context whose caller's stream is busy has not begun: another thread's
+    solve comes and goes meanwhile."""
+    s, other = solver(LATTICES["bend_24"]()), solver(LATTICES["bend_24"]())
+    for x in (s, other):
+        x.forward(tol=0, max_steps=100, check_every=100)
+    torch.cuda.synchronize()
+
+    def waits():
+        with torch.cuda.stream(torch.cuda.Stream()):
+            torch.cuda._sleep(2_000_000_000)  # about a second of one SM
+            other.forward(tol=0, max_steps=100, check_every=100)
+
+    t = threading.Thread(target=waits)
+    t.start()
+    time.sleep(0.2)
+    with torch.cuda.stream(torch.cuda.Stream()):
+        s.forward(tol=0, max_steps=100, check_every=100)
+    meanwhile = t.is_alive()
+    t.join()
+    assert meanwhile
+    s.close()
+    other.close()
