@@ -243,12 +243,12 @@ __device__ __forceinline__ Cell this_cell(int nx, int ny) {
     return c;
 }
 
-// the node of a thread of a plain step over widths off a multiple of 32: 256
-// consecutive nodes a block.  A row then starts anywhere in a 128-byte line;
-// tiles cut such lines between warps and leave lanes idle at every row's end.
-// 147 x 140 x 130: forward 76.4 -> 63.7 us, adjoint 76.5 -> 70.6; 129 x 96 x 80
-// coupled adjoint 37.7 -> 30.9.  Multiples of 32 keep the tiles (the divisions
-// cost the adjoint 2 % there).
+// the node of a thread of a plain step over widths off a multiple of 32, where
+// the lattice is large enough (make_step_geom): 256 consecutive nodes a block.  A
+// row then starts anywhere in a 128-byte line; tiles cut such lines between warps
+// and leave lanes idle at every row's end.  147 x 140 x 130: forward 76.4 -> 63.7 us,
+// adjoint 76.5 -> 70.6; 129 x 96 x 80 coupled adjoint 37.7 -> 30.9.  Multiples of 32
+// keep the tiles (the divisions cost the adjoint 2 % there).
 __device__ __forceinline__ Cell linear_cell(int nx, int ny, int nz) {
     const unsigned n = blockIdx.x * blockDim.x + threadIdx.x;  // below 2^31
     const unsigned row = n / (unsigned)nx;

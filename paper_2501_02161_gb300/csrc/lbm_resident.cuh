@@ -45,13 +45,14 @@
 // The node arithmetic is that of the one-step kernels, operation by operation.
 //
 // Measured, us a step (forward / adjoint) in launches of 500 steps against one
-// launch per step: 16^3 1.76 / 1.63 against 2.27 / 2.56, 32^3 2.23 / 2.22 against
-// 3.1 / 2.8, 64^3 FP32 4.38 / 4.33 against 5.65 / 5.73, temperature at
-// 192 x 48 x 24 1.84 / 1.76 against 3.29 / 3.46; 32^3 FP64, 300 steps of each,
-// 9.8 against 18.5 ms.  The set-up of a launch is about 25 us.  At 64^3 a block
-// issues 20000 warp instructions a step (5000 cycles of each scheduler) and takes
-// about 8500 cycles: what bounds it is the chain border - barrier - words -
-// barrier, of which the travel of the words is about 1500.
+// launch per step: 16^3 1.73 / 1.63 against 2.27 / 2.56, 32^3 2.23 / 2.21 against
+// 3.1 / 2.8, 64^3 FP32 4.40 / 4.36 against 5.65 / 5.73, temperature at
+// 192 x 48 x 24 1.78 / 1.70 against 4.13 / 4.38; 32^3 FP64 16.7 / 14.8 against
+// 29.5 / 31.5.  The set-up of a launch takes 20 us at 16^3 and 90 at 64^3 (the
+// nodes of a box are listed by one warp each), so short blocks do not go resident.
+// At 64^3 a block issues 20000 warp instructions a step (5000 cycles of each
+// scheduler) and takes about 8500 cycles: what bounds it is the chain border -
+// barrier - words - barrier, of which the travel of the words is about 1500.
 #pragma once
 
 #include "lbm_device.cuh"

@@ -107,9 +107,9 @@ ResPlan plan_boxes(int stencil, int storage, ResPhase ph, int nx, int ny, int nz
 }  // namespace
 
 // One block per SM; two for a temperature lattice whose boxes would have more
-// than one task per warp (192 x 48 x 24: 2.33 / 2.28 us a step against 2.60 /
-// 2.35 with one; the flow's boxes lose more to their larger surface: 64^3 6.5
-// against 5.3 us).
+// than one task per warp (192 x 48 x 24: 1.84 / 1.67 us a step against 2.06 /
+// 1.92 with one; the flow's boxes lose more to their larger surface: 64^3 5.28 /
+// 5.11 against 4.42 / 4.34).
 ResPlan resident_plan(int stencil, int storage, ResPhase ph, int nx, int ny, int nz) {
     int tasks = 0;
     ResPlan p = plan_boxes(stencil, storage, ph, nx, ny, nz, 1, tasks);

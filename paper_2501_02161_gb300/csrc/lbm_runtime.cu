@@ -304,10 +304,9 @@ ResPlan phase_plan(int stencil, int nx, int ny, int nz, int storage, bool therma
 }
 
 // The cuts of a context's phases (40 to 180 us of host time) and its inboxes (0.3
-// to 12.4 MB; 64^3 FP32: 7.7 beside 90): made for the first block that
-// may go resident, so that a context of a batch, which never does, neither waits
-// nor pays for them.  Without memory for the inboxes the context steps by
-// launches.
+// to 12.4 MB; 64^3 FP32: 7.7 beside 90) are made for the first block that may go
+// resident, so that a context of a batch, which never does, neither waits nor
+// pays for them.  Without memory for the inboxes the context steps by launches.
 void prepare_resident(lbm_ctx* c) {
     c->prepared = true;
     int sms = 0, coop = 0, smem = 0;
@@ -394,8 +393,6 @@ cudaError_t enqueue_block(lbm_ctx* c, int ph, int k, bool resident, cudaStream_t
 // launches (same results), which share the chip: 4 threads with a 96 x 48 x 24
 // heat sink each, 1000 steps: 11.8 ms, against 18.9 when one of them went
 // resident at a time; 2 with a 48^3 bend, 2000 steps: 9.6 against 12.3.
-// Whoever sees itself alone stays the only one that can until it has waited for
-// its launch: the next to come counts it.
 std::atomic<int> g_in_flight[64];
 
 struct InFlight {
@@ -407,11 +404,11 @@ struct InFlight {
     bool alone() const { return n == 1; }
 };
 
-// Held alone while a resident launch runs, shared while a launch per step is
-// enqueued: whoever comes meanwhile starts when the chip is free again.  Steps
-// of several contexts that had queued up behind a resident launch kept sharing
-// every SM from then on, their lattices evicting one another from L2 (8 threads
-// with a 64^3 bend each, 8000 steps: 456 ms for 379).
+// Held alone while a resident launch runs (so there is one at a time), shared
+// while the steps of a block are enqueued: whoever comes meanwhile starts when
+// the chip is free again.  Steps of several contexts that had queued up behind a
+// resident launch kept sharing every SM from then on, their lattices evicting
+// one another from L2 (8 threads with a 64^3 bend each, 8000 steps: 456 ms for 379).
 std::shared_mutex g_chip[64];
 
 // step numbers are 32 bits: start again from cleared inboxes before they run out
@@ -467,17 +464,19 @@ lbm_status run_block_sync(lbm_ctx* c, int ph, int k, const InFlight& solve) {
         // take long, or wait for what another thread does
         CUDA_TRY(cudaEventSynchronize(c->ev));
         std::unique_lock<std::shared_mutex> lock(chip);
-        if (run_block(c, ph, k, true) == LBM_OK) {
-            CUDA_TRY(cudaStreamSynchronize(c->stream));
-            if (c->hres[2] == 0.0) return LBM_OK;
-        } else {
-            (void)cudaGetLastError();
+        if (solve.alone()) {  // still
+            if (run_block(c, ph, k, true) == LBM_OK) {
+                CUDA_TRY(cudaStreamSynchronize(c->stream));
+                if (c->hres[2] == 0.0) return LBM_OK;
+            } else {
+                (void)cudaGetLastError();
+            }
+            // the launch was refused, or a wait gave up (the block's input is
+            // untouched and its reducing step was left out): the block runs
+            // again, a launch per step
+            ++c->gave_up;
+            CUDA_TRY(cudaMemsetAsync(c->sync + 1, 0, sizeof(unsigned), c->stream));
         }
-        // the launch was refused, or a wait gave up (the block's input is
-        // untouched and its reducing step was left out): the block runs
-        // again, a launch per step
-        ++c->gave_up;
-        CUDA_TRY(cudaMemsetAsync(c->sync + 1, 0, sizeof(unsigned), c->stream));
     }
     {
         std::shared_lock<std::shared_mutex> lock(chip);
@@ -1490,16 +1489,18 @@ lbm_status lbm_time_steps(lbm_ctx* c, int phase, int n, double* ms_per_step) {
     const long long m = (long long)n + (n & 1);  // an even count keeps the buffer parity
     const InFlight solve(c->device);
     float ms = 0.f;
-    bool began = false;
+    bool began = false, resident = false;
     // (the step numbers of all replays stay below the restart's threshold)
-    const bool resident = m <= 1 << 28 && resident_fits(c, phase, (int)(m / 2) - 1) && solve.alone();
-    if (resident) {
+    if (m <= 1 << 28 && resident_fits(c, phase, (int)(m / 2) - 1) && solve.alone()) {
         CUDA_TRY(cudaEventSynchronize(c->ev));
         std::unique_lock<std::shared_mutex> lock(g_chip[c->device & 63]);
-        st = time_replay(c, phase, m, true, &began, &ms);
-        if (st != LBM_OK && !began) {  // refused: nothing has run
-            (void)cudaGetLastError();
-            ++c->gave_up;
+        if (solve.alone()) {
+            st = time_replay(c, phase, m, true, &began, &ms);
+            resident = began;
+            if (!began) {  // refused: nothing has run
+                (void)cudaGetLastError();
+                ++c->gave_up;
+            }
         }
     }
     if (!began) st = time_replay(c, phase, m, false, &began, &ms);
