@@ -26,7 +26,9 @@
  *     lbm_set_stream (default: the legacy default stream), and that stream
  *     waits for the call's work before the call returns control to it.  Calls
  *     that report numbers (solves, lbm_get_*) synchronise.
- *   - A context is not thread-safe; distinct contexts are independent.
+ *   - A context is not thread-safe; distinct contexts are independent (a solve
+ *     or batch step may wait until another context's resident launch, a block
+ *     of steps of a lattice that fits on the chip, has ended).
  *
  * Node flag byte (bit-exact, identical in every call):
  *   bits 0-2  type: 0 FLUID, 1 WALL (full-way bounce-back, no collision,
