@@ -404,12 +404,20 @@ struct InFlight {
     bool alone() const { return n == 1; }
 };
 
-// Held alone while a resident launch runs (so there is one at a time), shared
-// while the steps of a block are enqueued: whoever comes meanwhile starts when
-// the chip is free again.  Steps of several contexts that had queued up behind a
-// resident launch kept sharing every SM from then on, their lattices evicting
-// one another from L2 (8 threads with a 64^3 bend each, 8000 steps: 456 ms for 379).
+// Held alone while a resident launch that fills the SMs runs, shared while the
+// steps of a block are enqueued: whoever comes meanwhile starts when the chip is
+// free again.  Steps of several contexts that had queued up behind a resident
+// launch kept sharing every SM from then on, their lattices evicting one another
+// from L2 (8 threads with a 64^3 bend each, 8000 steps: 456 ms for 379).
 std::shared_mutex g_chip[64];
+
+// A launch that leaves the registers for a block of one-step kernels (48 a
+// thread) on every SM lets others step beside it (4 threads with a 16^3 bend
+// each, 4000 steps: 11.3 ms, 12.0 when they waited for its end).
+bool fills_sm(const ResPlan& p, size_t real) {
+    const int regs = real == 8 ? 168 : 64;  // of k_resident
+    return p.threads * p.per_sm * regs + 256 * 48 > 65536;
+}
 
 // step numbers are 32 bits: start again from cleared inboxes before they run out
 lbm_status resident_tags(lbm_ctx* c, long long k) {
@@ -460,10 +468,13 @@ lbm_status run_block(lbm_ctx* c, int ph, int k, bool resident) {
 lbm_status run_block_sync(lbm_ctx* c, int ph, int k, const InFlight& solve) {
     std::shared_mutex& chip = g_chip[c->device & 63];
     if (resident_fits(c, ph, k - 1) && solve.alone()) {
-        // what the caller's stream holds comes first, without the lock: it may
-        // take long, or wait for what another thread does
-        CUDA_TRY(cudaEventSynchronize(c->ev));
-        std::unique_lock<std::shared_mutex> lock(chip);
+        std::unique_lock<std::shared_mutex> lock(chip, std::defer_lock);
+        if (fills_sm(c->plan[ph], c->rb)) {
+            // what the caller's stream holds comes first, without the lock: it may
+            // take long, or wait for what another thread does
+            CUDA_TRY(cudaEventSynchronize(c->ev));
+            lock.lock();
+        }
         if (solve.alone()) {  // still
             if (run_block(c, ph, k, true) == LBM_OK) {
                 CUDA_TRY(cudaStreamSynchronize(c->stream));
